@@ -115,9 +115,9 @@ bool factor_ok(int64_t n)
     return n == 1;
 }
 
-// Radix passes for a line of n points: the power-of-two part as evenly sized
-// radix-16/8/4/2 passes, then one pass per factor 3 and 5.
-std::vector<int> radix_plan(int64_t n)
+// Radix passes of a split-precision line of the generic family: the power-of-two part as evenly
+// sized radix-16/8/4/2 passes (radix 16 runs on the tensor cores), then one pass per factor 3 and 5.
+std::vector<int> split_radix_plan(int64_t n)
 {
     std::vector<int> r;
     int a = 0;
@@ -158,9 +158,12 @@ const KernelSet *lookup_kernels(int precision, int64_t n)
         // (which then compute the same) for the other specialised lengths
         if (const KernelSet *k = spec_kernels_split((int)n)) return k;
         if (const KernelSet *k = spec_kernels_f32((int)n)) return k;
+        if (n % 16 != 0)
+            if (const KernelSet *k = smooth_kernels_f32((int)n)) return k;
         return generic_kernels_split();
     }
     const KernelSet *k = precision == AFFT_F64 ? spec_kernels_f64((int)n) : spec_kernels_f32((int)n);
+    if (!k) k = precision == AFFT_F64 ? smooth_kernels_f64((int)n) : smooth_kernels_f32((int)n);
     if (k) return k;
     return precision == AFFT_F64 ? generic_kernels_f64() : generic_kernels_f32();
 }
@@ -176,7 +179,11 @@ void build_desc(int64_t n, const KernelSet *ks, StageDesc &d, std::vector<int> &
     const int base = (int)tm.size();
     std::vector<int> rad;
     if (!ks->generic) rad.assign(ks->radix, ks->radix + ks->npass);
-    else rad = radix_plan(n);
+    else if (ks == generic_kernels_split()) rad = split_radix_plan(n);
+    else {
+        int r[kMaxPasses];
+        rad.assign(r, r + std::max(0, radix_sequence(n, r)));
+    }
     d.npass = (int)rad.size();
     int ns = 1;
     for (int p = 0; p < d.npass; ++p) {
@@ -408,7 +415,8 @@ int plan_shapes(afft_plan *p)
         ap.pipe_slots = 0;
         if (ks->generic || !ks->pipe[PIPE_FWD_TMA] || ks->pipe_smem > max_smem) continue;
         for (int k = 0; k < PIPE_COUNT; ++k)
-            if (cudaFuncSetAttribute(ks->pipe[k], cudaFuncAttributeMaxDynamicSharedMemorySize, ks->pipe_smem) !=
+            if (ks->pipe[k] &&
+                cudaFuncSetAttribute(ks->pipe[k], cudaFuncAttributeMaxDynamicSharedMemorySize, ks->pipe_smem) !=
                 cudaSuccess)
                 return AFFT_ERR_CUDA;
         for (int k = 0; k < 2; ++k)
@@ -644,6 +652,8 @@ cudaError_t pipe_on_map(const AxisPlan &a, const CUtensorMap &map, bool tma, con
     return cudaLaunchKernel(fn, dim3(grid), dim3(a.ks->pipe_threads), args, (size_t)a.ks->pipe_smem, s);
 }
 
+// cudaErrorNotSupported, with nothing launched, when no kernel of the family loads these rows (the
+// caller then runs k_strided).
 template <typename V>
 cudaError_t strided_pipe(const AxisPlan &a, const V *in, V *out, const V *tw, long long outer, long long W,
                          int backward, unsigned *err, cudaStream_t s, int rev)
@@ -666,6 +676,7 @@ cudaError_t strided_pipe(const AxisPlan &a, const V *in, V *out, const V *tw, lo
         return cudaLaunchKernel(fn, dim3(grid), dim3(a.ks->pipe_threads), args, (size_t)a.ks->pipe_smem_rp, s);
     }
     const bool tma = encode_strided_map(&map, in, outer, a.desc.n, W, sizeof(V), a.ks->pipe_lines);
+    if (!tma && !a.ks->pipe[PIPE_FWD_CPASYNC]) return cudaErrorNotSupported;
     return pipe_on_map<V>(a, map, tma, in, out, tw, outer, W, backward, err, false, s, rev);
 }
 
@@ -674,7 +685,10 @@ template <typename V>
 cudaError_t strided(const AxisPlan &a, const V *in, V *out, const V *tw, long long outer, long long W,
                     int backward, cudaStream_t s, unsigned *err, int rev = 0)
 {
-    if (a.pipe) return strided_pipe<V>(a, in, out, tw, outer, W, backward, err, s, rev);
+    if (a.pipe) {
+        const cudaError_t e = strided_pipe<V>(a, in, out, tw, outer, W, backward, err, s, rev);
+        if (e != cudaErrorNotSupported) return e;
+    }
     StageDesc d = a.desc;
     d.rev = rev;
     tw += a.tw_base;
@@ -1727,10 +1741,12 @@ namespace {
 const char *strided_kernel_name(const afft_plan *p, int a, long long W)
 {
     const AxisPlan &ap = p->ax[a];
+    const size_t C = cplx_size(p->precision);
     if (!ap.pipe) return "k_strided";
-    if (cplx_size(p->precision) == 8 && (W % 2) == 1 && ap.rp_slots > 0 && ap.desc.n % 2 == 0 &&
-        ap.desc.n / 2 <= 256 && 2 * W >= ap.ks->pipe_lines + 2)
+    if (C == 8 && (W % 2) == 1 && ap.rp_slots > 0 && ap.desc.n % 2 == 0 && ap.desc.n / 2 <= 256 &&
+        2 * W >= ap.ks->pipe_lines + 2)
         return "k_strided_pipe_rp";
+    if (!ap.ks->pipe[PIPE_FWD_CPASYNC] && ((W * C) % 16 != 0 || W < ap.ks->pipe_lines)) return "k_strided";
     return "k_strided_pipe";
 }
 

@@ -4,7 +4,7 @@
 // process grid P0 = P1 = 1): batched 1-D FFTs along the contiguous axis N2,
 // then along N1, then along N0 (reverse order for the backward transform).
 // Each stage is one kernel launch.  A stage transforms every line of length n
-// with a Stockham autosort FFT made of radix-R passes (R in 16, 8, 4, 2, 3, 5);
+// with a Stockham autosort FFT made of radix-R passes (R in 16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2);
 // StageDesc carries that factorisation and the offsets of each pass's twiddle
 // table in the plan's device buffer.
 #pragma once
@@ -65,13 +65,53 @@ __host__ __device__ constexpr int bmax_for_radix(int r)
     return r >= 16 ? 1 : (r == 3 ? 5 : (r == 5 ? 3 : 16 / r));
 }
 
+// Radix passes for a line of n points of the generic family: the fewest passes of radices up to
+// 16 (every pass is a round trip through shared memory), and among those the smallest largest
+// radix, then the smallest sum, in descending order.  Writes at most kMaxPasses radices to r and
+// returns their number (0 for n == 1, -1 when n is not 2/3/5-smooth).
+inline int radix_sequence(long long n, int *r)
+{
+    static constexpr int kRadices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
+    if (n == 1) return 0;
+    struct Search {
+        int best[kMaxPasses], cur[kMaxPasses], best_max = 1 << 30, best_sum = 1 << 30;
+        void go(long long m, int left, int at, int hi, int sum)
+        {
+            if (left == 0) {
+                if (m != 1 || cur[0] > best_max || (cur[0] == best_max && sum >= best_sum)) return;
+                best_max = cur[0];
+                best_sum = sum;
+                for (int i = 0; i < at; ++i) best[i] = cur[i];
+                return;
+            }
+            for (int R : kRadices) {
+                if (R > hi || m % R != 0) continue;
+                cur[at] = R;
+                go(m / R, left - 1, at + 1, R, sum + R);
+            }
+        }
+    };
+    for (int k = 1; k <= 6; ++k) {   // lines of at most 4096 points need at most five (3125 = 5^5)
+        Search s;
+        s.go(n, k, 0, 16, 0);
+        if (s.best_sum < (1 << 30)) {
+            for (int i = 0; i < k; ++i) r[i] = s.best[i];
+            return k;
+        }
+    }
+    return -1;
+}
+
 // Rows per TMA box when a line of n rows is loaded in boxes of at most 256
 // rows: the largest divisor of n not above 256, so the boxes tile the line
-// exactly (used identically by the kernels and by the host's tensor maps).
+// exactly; an even one where n is even and takes several boxes, so that boxes of 64-byte
+// rows start 128-byte aligned in shared memory (used identically by the kernels and by the
+// host's tensor maps).
 __host__ __device__ constexpr int tma_box_rows(int n)
 {
-    int r = n < 256 ? n : 256;
-    while (r > 1 && n % r != 0) --r;
+    if (n <= 256) return n;
+    int r = 256;
+    while (r > 1 && (n % r != 0 || (n % 2 == 0 && r % 2 != 0))) --r;
     return r;
 }
 
@@ -144,6 +184,9 @@ struct KernelSet {
 // Specialised kernels for line length n, or nullptr.
 const KernelSet *spec_kernels_f32(int n);
 const KernelSet *spec_kernels_f64(int n);
+// The families of AFFT_SMOOTH_PLANS (the other 2/3/5-smooth lengths up to 1024), or nullptr.
+const KernelSet *smooth_kernels_f32(int n);
+const KernelSet *smooth_kernels_f64(int n);
 // Generic kernels (any n whose radix plan the host builds).
 const KernelSet *generic_kernels_f32();
 const KernelSet *generic_kernels_f64();

@@ -234,6 +234,73 @@ template <int S, typename V> struct Dft<5, S, V> {
     }
 };
 
+// R = A B with A and B coprime (Good-Thomas): with inputs read at (B a + A b) mod R and
+// outputs stored at the k with k = ka (mod A), k = kb (mod B), the length-R DFT is exactly the
+// A x B two-dimensional one, without twiddles: 6, 10, 12 and 15 cost no multiplication beyond
+// their factors' (radices 3 and 5 as separate passes would multiply every value once more and
+// cross shared memory once more).
+template <int A, int B, int S, typename V> struct DftCoprime {
+    __host__ __device__ static constexpr int crt(int ka, int kb)
+    {
+        int k = 0;
+        while (k % A != ka || k % B != kb) ++k;
+        return k;
+    }
+    static constexpr int eA = crt(1, 0), eB = crt(0, 1);
+    static __device__ __forceinline__ void run(V *v)
+    {
+        V t[A][B];
+#pragma unroll
+        for (int a = 0; a < A; ++a) {
+#pragma unroll
+            for (int b = 0; b < B; ++b) t[a][b] = v[(B * a + A * b) % (A * B)];
+            Dft<B, S, V>::run(t[a]);
+        }
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            V c[A];
+#pragma unroll
+            for (int a = 0; a < A; ++a) c[a] = t[a][b];
+            Dft<A, S, V>::run(c);
+#pragma unroll
+            for (int a = 0; a < A; ++a) v[(a * eA + b * eB) % (A * B)] = c[a];
+        }
+    }
+};
+template <int S, typename V> struct Dft<6, S, V> : DftCoprime<2, 3, S, V> {};
+template <int S, typename V> struct Dft<10, S, V> : DftCoprime<2, 5, S, V> {};
+template <int S, typename V> struct Dft<12, S, V> : DftCoprime<4, 3, S, V> {};
+template <int S, typename V> struct Dft<15, S, V> : DftCoprime<3, 5, S, V> {};
+
+// 9 = 3 x 3: A_q = DFT_3 over r1 of v[q + 3 r1]; A_q[s1] *= w_9^{q s1}; V[s1 + 3 s2] = DFT_3
+// over q of A_q[s1].
+template <int S, typename V> struct Dft<9, S, V> {
+    static __device__ __forceinline__ void run(V *v)
+    {
+        using T = typename RealOf<V>::T;
+        V a[3][3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+#pragma unroll
+            for (int r = 0; r < 3; ++r) a[q][r] = v[q + 3 * r];
+            Dft<3, S, V>::run(a[q]);
+        }
+        const T c1 = T(0.76604444311897803520), s1 = T(0.64278760968653932632);    // 40 degrees
+        const T c2 = T(0.17364817766693034885), s2 = T(0.98480775301220805937);    // 80 degrees
+        const T c4 = T(-0.93969262078590838405), s4 = T(0.34202014332566873304);   // 160 degrees
+        a[1][1] = cwc<S>(a[1][1], c1, s1);
+        a[1][2] = cwc<S>(a[1][2], c2, s2);
+        a[2][1] = cwc<S>(a[2][1], c2, s2);
+        a[2][2] = cwc<S>(a[2][2], c4, s4);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+            V c[3] = {a[0][s], a[1][s], a[2][s]};
+            Dft<3, S, V>::run(c);
+#pragma unroll
+            for (int t = 0; t < 3; ++t) v[s + 3 * t] = c[t];
+        }
+    }
+};
 
 // ------------------------------------------- float-float conversions -----
 

@@ -95,13 +95,15 @@ template <class P, typename V> struct PipeShape {
         for (int r : {Rs...}) m = r > m ? r : m;
         return m;
     }
+    template <int R0, int... Rs> __host__ __device__ static constexpr int first_radix(Seq<R0, Rs...>) { return R0; }
+    static constexpr bool first_pairs = pairs(first_radix(typename P::seq{}));
     // butterflies (or butterfly pairs) per thread; complex128 tiles (float-float arithmetic, twice
     // the registers per value) of plans without a radix-16 pass carry at most 8 values per thread,
     // for more warps per SM
     __host__ __device__ static constexpr int per_thread(int r)
     {
         return pairs(r) ? (16 / (2 * r) > 0 ? 16 / (2 * r) : 1)
-               : (sizeof(V) == 16 && max_radix(typename P::seq{}) <= 8) ? (8 / r > 1 ? 8 / r : 1)
+               : (sizeof(V) == 16 && P::df && max_radix(typename P::seq{}) <= 8) ? (8 / r > 1 ? 8 / r : 1)
                                                                       : bmax_for_radix(r);
     }
     __host__ __device__ static constexpr int units(int r) { return (pairs(r) ? lines / 2 : lines) * (P::n / r); }
@@ -138,10 +140,14 @@ template <class P, typename V> struct PipeShape {
     // odd-width complex64 rows read as row pairs (k_strided_pipe_rp): load buffers of two
     // [n/2][lines + 2] boxes, then the scratch tile and the mbarriers
     static constexpr int lw = lines + 2;
-    static constexpr int tile_rp = P::n * lw;
+    static constexpr int box_rp = ((P::n / 2) * lw * (int)sizeof(V) + 127) / 128 * 128 / (int)sizeof(V);  // second box's offset
+    static constexpr int tile_rp = 2 * box_rp;
     static constexpr int smem_rp = (2 * tile_rp + tile) * (int)sizeof(V) + 16 + tw_smem * 8;
-    static constexpr bool rp_ok = sizeof(V) == 8 && lines == 16 && P::n % 16 == 0 && P::n / 2 <= 256;
+    static constexpr bool rp_ok = sizeof(V) == 8 && lines == 16 && P::n % 2 == 0 && P::n / 2 <= 256;
     static constexpr int box_rows = tma_box_rows(P::n);
+    // TMA boxes must start 128-byte aligned in shared memory (625, 675 and 729 points in 64-byte
+    // rows do not: odd boxes)
+    static constexpr bool tma_ok = (box_rows * lines * (int)sizeof(V)) % 128 == 0 || box_rows == P::n;
     // split precision: the radix-16 passes' butterflies (tile / 16) fill whole 128-row blocks and
     // one 128-thread group per block covers them -- the tcgen05 pass runs unconditionally
     static constexpr bool tc_tile = sizeof(V) == 8 && (tile / 16) % 128 == 0 && threads % 128 == 0 &&
@@ -149,8 +155,16 @@ template <class P, typename V> struct PipeShape {
     // CTAs per SM the launch bounds ask for: two when two such CTAs' shared memory fits (tiles,
     // table and the tensor-core state, about 5 KB of static shared memory)
     static constexpr int min_blocks_split = 2 * (smem + 6 * 1024) <= 226 * 1024 ? 2 : 1;
-    static_assert((box_rows * lines * (int)sizeof(V)) % 128 == 0 || box_rows == P::n,
-                  "TMA boxes must start 128-byte aligned in shared memory");
+    // smooth lengths: as many CTAs as the tiles leave room for, at 64 registers a thread (a
+    // radix-16 butterfly of complex64) or 128 (complex128)
+    __host__ __device__ static constexpr int blocks_for(int bytes)
+    {
+        const int by_smem = 226 * 1024 / (bytes + 1024), by_regs = 65536 / (threads * (sizeof(V) == 8 ? 64 : 128));
+        const int b = by_smem < by_regs ? by_smem : by_regs;
+        return b < 1 ? 1 : (b > 4 ? 4 : b);
+    }
+    static constexpr int min_blocks = P::smooth ? blocks_for(smem) : 1;
+    static constexpr int min_blocks_rp = P::smooth ? blocks_for(smem_rp) : 1;
 };
 
 // ---------------------------------------------------------- pair passes ---
@@ -356,7 +370,8 @@ __device__ __forceinline__ bool pipe_df(Seq<R0, Rest...>, double2 *X, double2 *C
 // ---------------------------------------------------------------- kernel ---
 
 template <class P, int S, typename V, bool TMA, bool Split = false, bool Blocked = false>
-__global__ void __launch_bounds__(PipeShape<P, V>::threads, Split ? PipeShape<P, V>::min_blocks_split : 1)
+__global__ void __launch_bounds__(PipeShape<P, V>::threads, Split ? PipeShape<P, V>::min_blocks_split
+                                                                  : PipeShape<P, V>::min_blocks)
     k_strided_pipe(const V *__restrict__ in, V *out, const __grid_constant__ CUtensorMap tmap,
                    const V *__restrict__ tw, long long W, long long tiles_per_outer, long long ntiles,
                    unsigned *err, const void *twdf, const unsigned *mma, int rev)
@@ -470,7 +485,7 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, Split ? PipeShape<P,
             to.pair = PairGlobalOut{base, W, a, bcol, vec};
         }
         bool done = false;
-        if constexpr (std::is_same<V, double2>::value && P::npass >= 2) {
+        if constexpr (std::is_same<V, double2>::value && P::df) {
             if (twdf) {
                 TileOut<V, dcx> tdf;
                 tdf.single = GlobalColFixedOut<V, dcx>{to.single.base, to.single.W, to.single.col};
@@ -577,7 +592,7 @@ __device__ __forceinline__ void rp_passes(Seq<R0, Rest...>, float2 *X, float2 *C
 {
     constexpr int LG = Sh::lg, NT = Sh::threads, LW = Sh::lw;
     constexpr bool Last = sizeof...(Rest) == 0;
-    const float2 *A = X, *Bx = X + (N / 2) * LW;
+    const float2 *A = X, *Bx = X + Sh::box_rp;
     if constexpr (Sh::pairs(R0)) {
         constexpr int B = Sh::per_thread(R0);
         if constexpr (Last) pair_pass_rp<R0, S, N, LW, LG, NT, B>(A, Bx, out.pair);
@@ -605,7 +620,7 @@ __device__ __forceinline__ void rp_early_passes(Seq<R0, Rest...>, const float2 *
 {
     static_assert(sizeof...(Rest) >= 1, "the first pass must not be the last");
     constexpr int LG = Sh::lg, NT = Sh::threads, LW = Sh::lw;
-    const float2 *A = X, *Bx = X + (N / 2) * LW;
+    const float2 *A = X, *Bx = X + Sh::box_rp;
     if constexpr (Sh::pairs(R0))
         pair_pass_rp<R0, S, N, LW, LG, NT, Sh::per_thread(R0)>(A, Bx, PairSmemOut<LG>{C});
     else
@@ -621,7 +636,7 @@ __device__ __forceinline__ void rp_early_passes(Seq<R0, Rest...>, const float2 *
 // of 18 x n/2).  Early: the load buffer is released after the first pass
 // (two tile loads in flight during the other passes), as k_strided_pipe does.
 template <class P, int S, bool Early = false>
-__global__ void __launch_bounds__(PipeShape<P, float2>::threads, 1)
+__global__ void __launch_bounds__(PipeShape<P, float2>::threads, PipeShape<P, float2>::min_blocks_rp)
     k_strided_pipe_rp(const float2 *__restrict__, float2 *out, const __grid_constant__ CUtensorMap tmap,
                       const float2 *__restrict__ tw, long long W, long long tiles_per_outer, long long ntiles,
                       unsigned *err, const void *, const unsigned *, int rev)
@@ -630,7 +645,7 @@ __global__ void __launch_bounds__(PipeShape<P, float2>::threads, 1)
     using Sh = PipeShape<P, V>;
     constexpr int N = P::n, LINES = Sh::lines, LW = Sh::lw, TILE_RP = Sh::tile_rp;
     constexpr unsigned BOX_BYTES = (N / 2) * LW * sizeof(V);
-    static_assert(Sh::rp_ok, "row-pair tiles: 16 complex64 columns, n a multiple of 16, at most 512");
+    static_assert(Sh::rp_ok, "row-pair tiles: 16 complex64 columns, n even, at most 512");
     extern __shared__ __align__(1024) unsigned char pipe_smem_raw[];
     V *const buf0 = reinterpret_cast<V *>(pipe_smem_raw);   // load buffer b at buf0 + b * TILE_RP
     V *const scratch = buf0 + 2 * TILE_RP;
@@ -658,7 +673,7 @@ __global__ void __launch_bounds__(PipeShape<P, float2>::threads, 1)
         fence_async_shared();
         mbar_expect_tx(&bars[b], 2 * BOX_BYTES);
         tma_load_3d(buf0 + b * TILE_RP, &tmap, (int)c0, 0, (int)o, &bars[b]);
-        tma_load_3d(buf0 + b * TILE_RP + (N / 2) * LW, &tmap, (int)(W + c0 - 1), 0, (int)o, &bars[b]);
+        tma_load_3d(buf0 + b * TILE_RP + Sh::box_rp, &tmap, (int)(W + c0 - 1), 0, (int)o, &bars[b]);
     };
 
     // Without Early the next tile's load is issued once this one has landed.
@@ -886,9 +901,29 @@ template <class F, typename V> KernelSet kernel_set(int n, int npass, const int 
     if constexpr (!F::generic) {
         // n = 1024 would need 64-byte tile rows to double-buffer; measured slower than the
         // single-buffered kernel with the same rows, so it keeps the non-pipelined kernel.
-        if constexpr (F::plan::npass > 0 && F::plan::n <= 1024) {
+        if constexpr (F::plan::smooth) {
+            // TMA tiles alone (rows that no tensor map covers take k_strided), one row-pair form
+            // (early release when the first pass works on column pairs), no blocked layout and no
+            // fused Poisson operator: what the generic kernels served before had none of these
             using P = typename F::plan;
             using Sh = PipeShape<P, V>;
+            if constexpr (Sh::tma_ok) {
+                k.pipe[PIPE_FWD_TMA] = (const void *)k_strided_pipe<P, -1, V, true>;
+                k.pipe[PIPE_BWD_TMA] = (const void *)k_strided_pipe<P, +1, V, true>;
+                k.pipe_lines = Sh::lines;
+                k.pipe_threads = Sh::threads;
+                k.pipe_smem = Sh::smem;
+                if constexpr (Sh::rp_ok) {
+                    constexpr bool early = P::npass >= 2 && Sh::first_pairs;
+                    k.pipe_rp[0] = (const void *)k_strided_pipe_rp<P, -1, early>;
+                    k.pipe_rp[1] = (const void *)k_strided_pipe_rp<P, +1, early>;
+                    k.pipe_smem_rp = Sh::smem_rp;
+                }
+            }
+        } else if constexpr (F::plan::npass > 0 && F::plan::n <= 1024) {
+            using P = typename F::plan;
+            using Sh = PipeShape<P, V>;
+            static_assert(Sh::tma_ok, "TMA boxes must start 128-byte aligned in shared memory");
             k.pipe[PIPE_FWD_TMA] = (const void *)k_strided_pipe<P, -1, V, true, F::split>;
             k.pipe[PIPE_FWD_CPASYNC] = (const void *)k_strided_pipe<P, -1, V, false, F::split>;
             k.pipe[PIPE_BWD_TMA] = (const void *)k_strided_pipe<P, +1, V, true, F::split>;

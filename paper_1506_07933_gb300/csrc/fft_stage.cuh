@@ -110,7 +110,17 @@ template <int... Rs> struct Seq {};
 template <int N, int... Rs> struct LinePlan {
     static constexpr int n = N;
     static constexpr int npass = sizeof...(Rs);
+    static constexpr bool df = npass >= 2;   // complex128 lines compute in float-float (needs two passes)
+    static constexpr bool smooth = false;
     using seq = Seq<Rs...>;
+};
+
+// A length of AFFT_SMOOTH_PLANS: complex128 lines compute in FP64 (these lengths always did, and
+// float-float would give up the last four of its 52 bits), and only the kernels a plan can reach
+// are instantiated (see kernel_set).
+template <int N, int... Rs> struct SmoothPlan : LinePlan<N, Rs...> {
+    static constexpr bool df = false;
+    static constexpr bool smooth = true;
 };
 
 // One pass of a specialised sequence: radix_pass, or with Split (complex64
@@ -207,9 +217,9 @@ __device__ __forceinline__ bool df_stage(const CT *tw, int lines, const Map &map
     return df_stage_impl<P, S, LastToSmem>(typename P::seq{}, tw, lines, map, src, sm, dst, bad);
 }
 
-// Specialised FP64 kernels with at least two passes compute in float-float.
+// FP64 kernels of plans with df compute in float-float.
 template <class F, typename V> struct UseDf {
-    static constexpr bool value = !F::generic && std::is_same<V, double2>::value && F::plan::npass >= 2;
+    static constexpr bool value = !F::generic && std::is_same<V, double2>::value && F::plan::df;
 };
 
 // ------------------------------------------------- generic pass sequence ----
@@ -253,7 +263,12 @@ __device__ __forceinline__ void smem_pass_any(int R, V *sm, int n, int Ns, const
         else
             smem_pass<16, S, Rows>(sm, n, Ns, tw, lines, log2_lines);
         break;
+    case 15: smem_pass<15, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+    case 12: smem_pass<12, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+    case 10: smem_pass<10, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+    case 9: smem_pass<9, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 8: smem_pass<8, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+    case 6: smem_pass<6, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 4: smem_pass<4, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 2: smem_pass<2, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 3: smem_pass<3, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
@@ -488,11 +503,12 @@ __device__ __forceinline__ void r2c_post(const Tile &tile, V *o, const CT *post_
 // t owns the bin pair k = t mod M/2 (k and M - k) of lines t div M/2, +step,
 // ..., so its twiddle is loaded once and no index is divided; k = 0 also
 // writes X[M] and X[M/2] = conj Z[M/2] (E = Re Z, O = Im Z, w^{M/2} = -i).
-// Returns false, doing nothing, when the CTA size does not fit.
+// Returns false, doing nothing, when M is odd (bin M/2 is then no bin of its own) or the CTA size
+// does not fit.
 template <int M, typename V, typename CT, class Tile>
 __device__ __forceinline__ bool r2c_post_fixed_k(const Tile &tile, V *o, const CT *post_tw, int ld, int valid)
 {
-    if constexpr (M < 2) {
+    if constexpr (M % 2 != 0) {
         return false;
     } else {
         using T = typename RealOf<CT>::T;
@@ -713,5 +729,31 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
     X(16, 16) X(32, 16, 2) X(48, 16, 3) X(64, 16, 4) X(80, 16, 5) X(96, 16, 3, 2) X(128, 16, 8)     \
     X(160, 16, 5, 2) X(192, 16, 4, 3) X(256, 16, 16) X(384, 16, 8, 3) X(512, 16, 16, 2)             \
     X(1024, 16, 16, 4) X(2048, 16, 16, 8) X(4096, 16, 16, 16)
+
+// The other 2/3/5-smooth lengths up to 1024 (3, 5, 6, 9, ... 1000): radix sequences as
+// radix_sequence() picks them, the fewest passes first.  A line of the generic kernels costs one
+// shared-memory round trip per pass plus two to stage the tile, with run-time lengths in every
+// index and one tile per CTA in flight.  Measured, generic kernels -> these: a c2c stage of 243^3
+// complex64 304-367 -> 66-75 us (230 MB through HBM: 34 us), the N1 stage of 320 x 300 x 500 r2c
+// 393 -> 91 us, its r2c stage 469 -> 147 us; complex128 (bound by the FP64 pipe) 250 -> 186-232 us
+// a stage of 180 x 200 x 216 r2c, from fewer inter-pass twiddles.
+// Above 1024 points lines are rare enough to stay with the generic kernels.  (Four groups: one
+// translation unit each per precision.)
+#define AFFT_SMOOTH_PLANS_A(X)                                                                      \
+    X(18, 6, 3) X(20, 5, 4) X(36, 6, 6) X(81, 9, 9) X(90, 10, 9) X(200, 8, 5, 5) X(243, 9, 9, 3)    \
+    X(250, 10, 5, 5) X(320, 8, 8, 5) X(450, 10, 9, 5) X(500, 10, 10, 5) X(625, 5, 5, 5, 5)          \
+    X(640, 10, 8, 8) X(675, 15, 9, 5) X(750, 15, 10, 5) X(810, 10, 9, 9)
+#define AFFT_SMOOTH_PLANS_B(X)                                                                      \
+    X(6, 6) X(9, 9) X(27, 9, 3) X(30, 6, 5) X(72, 9, 8) X(125, 5, 5, 5) X(135, 15, 9)               \
+    X(180, 15, 12) X(216, 6, 6, 6) X(240, 16, 15) X(270, 9, 6, 5) X(432, 9, 8, 6)                   \
+    X(480, 10, 8, 6) X(540, 10, 9, 6) X(729, 9, 9, 9) X(864, 12, 9, 8) X(960, 12, 10, 8)
+#define AFFT_SMOOTH_PLANS_C(X)                                                                      \
+    X(3, 3) X(12, 12) X(25, 5, 5) X(45, 9, 5) X(50, 10, 5) X(75, 15, 5) X(108, 12, 9)               \
+    X(225, 15, 15) X(288, 8, 6, 6) X(324, 9, 6, 6) X(360, 9, 8, 5) X(400, 10, 8, 5)                 \
+    X(486, 9, 9, 6) X(648, 9, 9, 8) X(720, 10, 9, 8) X(900, 10, 10, 9) X(972, 12, 9, 9)
+#define AFFT_SMOOTH_PLANS_D(X)                                                                      \
+    X(5, 5) X(10, 10) X(15, 15) X(40, 8, 5) X(54, 9, 6) X(100, 10, 10) X(144, 12, 12)               \
+    X(150, 15, 10) X(162, 9, 6, 3) X(300, 10, 6, 5) X(375, 15, 5, 5) X(405, 9, 9, 5)                \
+    X(576, 9, 8, 8) X(600, 10, 10, 6) X(768, 12, 8, 8) X(800, 10, 10, 8) X(1000, 10, 10, 10)
 
 }  // namespace afft

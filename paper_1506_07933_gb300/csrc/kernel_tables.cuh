@@ -26,3 +26,8 @@ template <size_t K> const KernelSet *find_set(const KernelSet (&table)[K], int n
 #define AFFT_KERNEL_SET(V, SPLIT, N, ...)                                                            \
     afft::kernel_set<afft::Spec<afft::LinePlan<N, ##__VA_ARGS__>, SPLIT>, V>(                         \
         N, afft::LinePlan<N, ##__VA_ARGS__>::npass, afft::RadicesOf<afft::LinePlan<N, ##__VA_ARGS__>>::value),
+
+// The same for a SmoothPlan.
+#define AFFT_SMOOTH_SET(V, N, ...)                                                                   \
+    afft::kernel_set<afft::Spec<afft::SmoothPlan<N, ##__VA_ARGS__>>, V>(                              \
+        N, afft::LinePlan<N, ##__VA_ARGS__>::npass, afft::RadicesOf<afft::LinePlan<N, ##__VA_ARGS__>>::value),

@@ -1,0 +1,14 @@
+// kernels_smooth_f64_a.cu -- the double2 families of the line lengths in AFFT_SMOOTH_PLANS_A.
+#include "kernel_tables.cuh"
+
+namespace afft {
+
+#define AFFT_X(N, ...) AFFT_SMOOTH_SET(double2, N, ##__VA_ARGS__)
+
+const KernelSet *smooth_kernels_f64_a(int n)
+{
+    static const KernelSet table[] = {AFFT_SMOOTH_PLANS_A(AFFT_X)};
+    return find_set(table, n);
+}
+
+}  // namespace afft

@@ -67,22 +67,6 @@ bool smooth(int64_t n)
     return n == 1;
 }
 
-// Radix sequence for a length without specialised kernels (the generic
-// kernels accept any sequence whose product is n): radix-16/8/4/2 passes of
-// balanced size, then 3s, then 5s.
-int radix_plan(int64_t n, int *r)
-{
-    int k = 0, a = 0;
-    while (n % 2 == 0) { n /= 2; ++a; }
-    if (a > 0) {
-        const int passes = (a + 3) / 4;
-        for (int i = 0; i < passes; ++i) r[k++] = 1 << (a / passes + (i < a % passes ? 1 : 0));
-    }
-    while (n % 3 == 0) { n /= 3; r[k++] = 3; }
-    while (n % 5 == 0) { n /= 5; r[k++] = 5; }
-    return k;
-}
-
 struct Axis {
     StageDesc d;
     const KernelSet *ks;
@@ -110,6 +94,7 @@ void describe(int64_t n, int precision, Axis &a, int &tw_count)
 {
     std::memset(&a.d, 0, sizeof a.d);
     a.ks = precision == AFFT_F64 ? spec_kernels_f64((int)n) : spec_kernels_f32((int)n);
+    if (!a.ks) a.ks = precision == AFFT_F64 ? smooth_kernels_f64((int)n) : smooth_kernels_f32((int)n);
     if (!a.ks) a.ks = precision == AFFT_F64 ? generic_kernels_f64() : generic_kernels_f32();
     a.d.n = (int)n;
     int rad[kMaxPasses];
@@ -118,7 +103,7 @@ void describe(int64_t n, int precision, Axis &a, int &tw_count)
         np = a.ks->npass;
         for (int i = 0; i < np; ++i) rad[i] = a.ks->radix[i];
     } else {
-        np = radix_plan(n, rad);
+        np = radix_sequence(n, rad);
     }
     a.d.npass = np;
     a.tw_base = tw_count;

@@ -1,0 +1,51 @@
+"""Line lengths with prime factors 2, 3, 5 that are not in the main table (AFFT_SMOOTH_PLANS): every
+length up to 1024 on every axis and in every kernel it can take, against the FP64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1506_07933_gb300 import afft, synth
+
+pytestmark = pytest.mark.gpu
+
+
+def smooth(n):
+    for p in (2, 3, 5):
+        while n % p == 0:
+            n //= p
+    return n == 1
+
+
+MAIN = {2, 4, 8, 16, 24, 32, 48, 60, 64, 80, 96, 120, 128, 160, 192, 256, 384, 512, 1024}
+LENGTHS = [n for n in range(2, 1025) if smooth(n) and n not in MAIN]
+# five-smooth lengths of the generic kernels with radices 6, 9, 10, 12 and 15 among their passes
+GENERIC = [1080, 1125, 1458, 1728, 3125]
+# FP64 lines of these lengths compute in FP64: a length-n FFT of log2(n) <= 12 levels stays within a
+# few eps sqrt(log2 n), far below the float-float kernels' 1e-14
+TOL = {"f32": 2e-6, "f64": 4e-15}
+CDT = {"f32": np.complex64, "f64": np.complex128}
+RDT = {"f32": np.float32, "f64": np.float64}
+
+
+def check(shape, kind, prec, seed):
+    make = synth.uniform_complex if kind == "c2c" else synth.uniform_real
+    x = make(shape, seed).astype((CDT if kind == "c2c" else RDT)[prec])
+    ref = oracle.c2c(x, -1, "fft") if kind == "c2c" else oracle.r2c(x)
+    with afft.Plan(shape, kind, prec) as p:
+        X = p.forward(torch.from_numpy(x).cuda())
+        y = p.backward(torch.from_numpy(ref.astype(CDT[prec])).cuda())
+        torch.cuda.synchronize()
+        assert p.device_status() == 0
+    assert oracle.rel_l2(X.cpu().numpy(), ref) <= TOL[prec], (shape, kind, prec, "forward")
+    assert oracle.rel_l2(y.cpu().numpy(), x) <= TOL[prec], (shape, kind, prec, "backward")
+
+
+@pytest.mark.parametrize("n", LENGTHS + GENERIC)
+def test_length_on_every_axis(n):
+    for prec in ("f32", "f64"):
+        check((n, 4, 10), "c2c", prec, n)          # N0: TMA tiles, the last one ragged
+        check((2, n, 25), "c2c", prec, n + 1)      # N1: rows of odd width (row pairs, or no tensor map)
+        check((3, 5, n), "c2c", prec, n + 2)       # N2: whole lines
+        check((3, n, 36), "r2c", prec, n + 3)      # N1 of an r2c plan: 19 bins per row
+        check((2, 5, 2 * n), "r2c", prec, n + 4)   # half-length lines of r2c and c2r
