@@ -192,8 +192,9 @@ void build_desc(int64_t n, const KernelSet *ks, StageDesc &d, std::vector<int> &
         d.ns[p] = ns;
         d.tw_off[p] = (int)tm.size() - base;
         if (ns > 1) {
-            for (int k = 0; k < ns; ++k)
-                for (int r = 1; r < R; ++r) {
+            // r-major: the threads of a contiguous line take consecutive k, one run of the table per r
+            for (int r = 1; r < R; ++r)
+                for (int k = 0; k < ns; ++k) {
                     tm.push_back((int)(((long long)r * k) % ((long long)R * ns)));
                     tl.push_back(R * ns);
                 }
@@ -248,7 +249,7 @@ bool shape_strided(const StageDesc &d, long long outer, long long W, size_t elem
 // even_lines: an even count where possible, so that every CTA's run of lines of
 // an odd number of complex64 elements starts 16-byte aligned (the c2r kernel
 // then stages it with 16-byte copies).
-bool shape_contig(const StageDesc &d, long long nlines, size_t elem, int max_threads, size_t max_smem,
+bool shape_contig(const StageDesc &d, const KernelSet *ks, long long nlines, size_t elem, size_t max_smem,
                   Launch &L, int target = 0, bool even_lines = false)
 {
     if (target <= 0) target = elem == 8 ? 4096 : 2048;
@@ -258,9 +259,8 @@ bool shape_contig(const StageDesc &d, long long nlines, size_t elem, int max_thr
     const int row = (int)(128 / elem);
     for (;;) {
         const int thr = required_threads(d, lines);
-        const size_t pts = ((size_t)lines * d.n + row - 1) / row * row;
-        const size_t smem = pts * elem;
-        if (thr <= max_threads && smem <= max_smem) {
+        const size_t smem = (size_t)contig_tile_elems(lines * d.n, row, ks->contig_pad) * elem;
+        if (thr <= ks->max_threads && smem <= max_smem) {
             L.lines = lines;
             L.log2_lines = 0;
             L.threads = thr;
@@ -485,7 +485,7 @@ int plan_shapes(afft_plan *p)
         AxisPlan &ap = p->ax[a];
         bool ok;
         if (a == 2 && !f.on)
-            ok = shape_contig(z.desc, B * n0 * n1, elem, z.ks->max_threads, budget(z), z.launch, 0,
+            ok = shape_contig(z.desc, z.ks, B * n0 * n1, elem, budget(z), z.launch, 0,
                               p->kind == AFFT_R2C && (nh & 1));
         else ok = shape_strided(ap.desc, outer[a], width[a] * (f.on ? f.na : 1), elem, ap.ks->max_threads,
                                 budget(ap), ap.launch);
@@ -1228,7 +1228,7 @@ bool reshape_contig(afft_plan *p, int target)
     const size_t budget = z.ks->generic ? (size_t)max_smem : (size_t)std::min(max_smem, 112 * 1024);
     Launch L;
     const bool even = p->kind == AFFT_R2C && ((p->n[2] / 2 + 1) & 1);
-    if (!shape_contig(z.desc, p->batch * p->n[0] * p->n[1], sizeof(V), z.ks->max_threads, budget, L, target, even))
+    if (!shape_contig(z.desc, z.ks, p->batch * p->n[0] * p->n[1], sizeof(V), budget, L, target, even))
         return false;
     z.launch = L;
     p->contig_target = target;

@@ -115,6 +115,14 @@ __host__ __device__ constexpr int tma_box_rows(int n)
     return r;
 }
 
+// Elements of a contiguous stage's shared tile of `points` values, 128-byte rows of `row` values
+// (pad: one spare value after each row, see SmemTile), rounded up to whole rows.
+__host__ __device__ constexpr int contig_tile_elems(int points, int row, bool pad)
+{
+    const int e = pad ? points + points / row + 1 : points;
+    return (e + row - 1) / row * row;
+}
+
 struct Launch {
     int lines;                     // lines (columns) per CTA
     int log2_lines;                // log2(lines) for the strided stage (lines is a power of 2)
@@ -157,6 +165,7 @@ struct KernelSet {
     const void *fn[KS_COUNT];
     int max_threads;               // largest CTA the kernels were compiled for
     bool generic;
+    bool contig_pad;               // the contiguous kernels pad their shared tile (contig_tile_elems)
     const void *pipe[PIPE_COUNT];  // null when the family has no pipelined strided kernel
     const void *pipe_blk[2];       // its blocked-row TMA variants ([0] forward, [1] backward)
     // generic family only: second half of a four-step line, (const V *in, V *out,

@@ -217,10 +217,10 @@ __device__ __forceinline__ void pair_pass(const float2 *src, const float2 *__res
             }
             const int k = j % Ns;
             if (Ns > 1) {
-                const float2 *t = tw + k * (R - 1);
+                const float2 *t = tw + k;
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    const float2 w = tw_ld<TwSmem>(t + r - 1);
+                    const float2 w = tw_ld<TwSmem>(t + (r - 1) * Ns);
                     lo[b][r] = ctw<S>(lo[b][r], w);
                     hi[b][r] = ctw<S>(hi[b][r], w);
                 }
@@ -893,6 +893,7 @@ template <class F, typename V> KernelSet kernel_set(int n, int npass, const int 
     k.fn[KS_C2R] = (const void *)k_c2r<F, V>;
     k.max_threads = F::template threads<V>();
     k.generic = F::generic;
+    k.contig_pad = F::plan::pad;
     if constexpr (F::generic) {
         k.four[0] = (const void *)k_fourstep<-1, V, F::split>;
         k.four[1] = (const void *)k_fourstep<+1, V, F::split>;

@@ -83,7 +83,7 @@ __device__ __noinline__ void q_r2c(const QGroup &g, unsigned plane, unsigned k, 
     const int valid = min(g.zlines, g.n1 - (int)k * g.zlines);
     // the input is the caller's array, written before the launch: plain loads
     const GlobalLines<float2> src{reinterpret_cast<const float2 *>(g.in) + b0 * M, M, valid};
-    const SmemLines<float2> tile{sm, M};
+    const SmemTile<float2, M, P::pad> tile{sm};
     run_plan<P, -1, true>(g.tw[2], g.zlines, MapButterflyFast{}, src, tile, tile);
     __syncthreads();
     float2 *o = reinterpret_cast<float2 *>(g.out) + b0 * (M + 1);
@@ -125,10 +125,10 @@ __device__ __noinline__ void q_c2r(const QGroup &g, unsigned plane, unsigned k, 
         __syncthreads();
         const C2RPre<float2> sx{sm, g.post, M, M + 1, valid};
         run_plan_staged<P, +1>(typename P::seq{}, g.tw[2], g.zlines, MapButterflyFast{}, sx,
-                               SmemLines<float2>{sm, M}, dst);
+                               SmemTile<float2, M, P::pad>{sm}, dst);
     } else {
         const C2RPre<float2, float2, true> sx{xin, g.post, M, M + 1, valid};
-        run_plan<P, +1, false>(g.tw[2], g.zlines, MapButterflyFast{}, sx, SmemLines<float2>{sm, M}, dst);
+        run_plan<P, +1, false>(g.tw[2], g.zlines, MapButterflyFast{}, sx, SmemTile<float2, M, P::pad>{sm}, dst);
     }
 }
 

@@ -108,11 +108,11 @@ __device__ __forceinline__ void mma16_pass(int n, int Ns, const float2 *__restri
 #pragma unroll
             for (int t = 0; t < 4; ++t) x[t] = src(l, j + (q + 4 * t) * nb);
             if (Ns > 1) {
-                const float2 *w = tw + (j % Ns) * 15;
+                const float2 *w = tw + j % Ns;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     const int r = q + 4 * t;
-                    if (r > 0) x[t] = ctw<S>(x[t], ldgc(w + r - 1));
+                    if (r > 0) x[t] = ctw<S>(x[t], ldgc(w + (r - 1) * Ns));
                 }
             }
         }

@@ -81,11 +81,11 @@ __device__ __forceinline__ void radix_pass(int n, int Ns, const V *__restrict__ 
             lb[b] = l;
             jb[b] = j;
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[b][r] = src(l, j + r * nb);
+            for (int r = 0; r < R; ++r) v[b][r] = tile_ld(src, l, j, r * nb);
             if (Ns > 1) {
-                const V *t = tw + (j % Ns) * (R - 1);
+                const V *t = tw + j % Ns;
 #pragma unroll
-                for (int r = 1; r < R; ++r) v[b][r] = ctw<S>(v[b][r], tw_ld<TwSmem>(t + r - 1));
+                for (int r = 1; r < R; ++r) v[b][r] = ctw<S>(v[b][r], tw_ld<TwSmem>(t + (r - 1) * Ns));
             }
             Dft<R, S, V>::run(v[b]);
         }
@@ -98,7 +98,7 @@ __device__ __forceinline__ void radix_pass(int n, int Ns, const V *__restrict__ 
             const int k = j % Ns;
             const int o = (j - k) * R + k;
 #pragma unroll
-            for (int r = 0; r < R; ++r) dst(lb[b], o + r * Ns, cnorm(v[b][r]));
+            for (int r = 0; r < R; ++r) tile_st(dst, lb[b], o, r * Ns, cnorm(v[b][r]));
         }
     }
 }
@@ -112,6 +112,9 @@ template <int N, int... Rs> struct LinePlan {
     static constexpr int npass = sizeof...(Rs);
     static constexpr bool df = npass >= 2;   // complex128 lines compute in float-float (needs two passes)
     static constexpr bool smooth = false;
+    template <int R0, int... R> __host__ __device__ static constexpr bool pad_for(Seq<R0, R...>) { return R0 % 4 == 0; }
+    __host__ __device__ static constexpr bool pad_for(Seq<>) { return false; }
+    static constexpr bool pad = pad_for(Seq<Rs...>{});   // contiguous tiles: see SmemTile
     using seq = Seq<Rs...>;
 };
 
@@ -341,6 +344,9 @@ struct GenericSplit {
     static constexpr int min_blocks = 1;
 };
 
+// The shared tile of a specialised family's contiguous kernels.
+template <typename V, class F> using ContigTile = SmemTile<V, F::plan::n, F::plan::pad>;
+
 // ------------------------------------------------------------- kernels ------
 
 // Strided axis: lines run along a [outer][n][W] slab with stride W; the CTA
@@ -406,11 +412,11 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
                 DfFlags bad;
                 const GlobalLines<V, dcx> sdf{in0, n, valid, &bad};
                 const GlobalLinesOut<V, dcx> ddf{out0, n, valid, dfl(scale)};
-                const SmemLines<dcx> tdf{reinterpret_cast<dcx *>(sm), n};
+                const ContigTile<dcx, F> tdf{reinterpret_cast<dcx *>(sm)};
                 if (df_stage<typename F::plan, S, false>((const dcx *)d.twdf, lines, map, sdf, tdf, ddf, bad)) return;
             }
         }
-        const SmemLines<V> tile{sm, n};
+        const ContigTile<V, F> tile{sm};
         if constexpr (F::split && std::is_same<V, float2>::value) {
             // split precision: radix-16 passes on tcgen05 (fft_tc.cuh) where the CTA allows
             tc_setup(reinterpret_cast<const unsigned char *>(d.mma) + kMmaTableWords * 4 + (S < 0 ? 0 : kTcBBytes),
@@ -551,7 +557,6 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
     const long long b0 = stage_order(blockIdx.x, gridDim.x, d.rev) * lines;
     const int valid = (int)min((long long)lines, nlines - b0);
     const GlobalLines<V> src{reinterpret_cast<const V *>(in) + b0 * M, M, valid};
-    const SmemLines<V> tile{sm, M};
     const MapButterflyFast map{};
     const int ld = d.ld > 0 ? d.ld : M + 1;  // output line stride (d.ld > 0: lines further apart)
     V *o = out + b0 * ld;
@@ -559,7 +564,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
         if (d.twdf) {
             DfFlags bad;
             const GlobalLines<V, dcx> sdf{reinterpret_cast<const V *>(in) + b0 * M, M, valid, &bad};
-            const SmemLines<dcx> tdf{reinterpret_cast<dcx *>(sm), M};
+            const ContigTile<dcx, F> tdf{reinterpret_cast<dcx *>(sm)};
             if (df_stage<typename F::plan, -1, true>((const dcx *)d.twdf, lines, map, sdf, tdf, tdf, bad)) {
                 __syncthreads();
                 // (float-float tiles keep the general loop: the fixed-bin form measured no faster)
@@ -570,13 +575,20 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
     }
     // (the input is read from global memory in the first pass: staging it in shared memory as
     // k_c2r does measured 12% slower here, the 16 loads of a thread being in flight together)
-    if constexpr (F::generic) run_generic<-1, false, true, F::split>(d, tw, sm, lines, 0, map, src, tile);
-    else run_plan<typename F::plan, -1, true, F::split>(tw, lines, map, src, tile, tile, d.mma);
-    __syncthreads();
-    if constexpr (!F::generic && sizeof(V) == 8) {
-        if (r2c_post_fixed_k<F::plan::n, V, V>(tile, o, post_tw, ld, valid)) return;
+    if constexpr (F::generic) {
+        const SmemLines<V> tile{sm, M};
+        run_generic<-1, false, true, F::split>(d, tw, sm, lines, 0, map, src, tile);
+        __syncthreads();
+        r2c_post<V, V>(tile, o, post_tw, M, ld, valid);
+    } else {
+        const ContigTile<V, F> tile{sm};
+        run_plan<typename F::plan, -1, true, F::split>(tw, lines, map, src, tile, tile, d.mma);
+        __syncthreads();
+        if constexpr (sizeof(V) == 8) {
+            if (r2c_post_fixed_k<F::plan::n, V, V>(tile, o, post_tw, ld, valid)) return;
+        }
+        r2c_post<V, V>(tile, o, post_tw, M, ld, valid);
     }
-    r2c_post<V, V>(tile, o, post_tw, M, ld, valid);
     (void)sizeof(T);
 }
 
@@ -618,7 +630,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
                     return;
                 }
                 const C2RPre<V> sx{sm, post_tw, M, M + 1, valid};
-                run_plan_staged<typename F::plan, +1>(typename F::plan::seq{}, tw, lines, map, sx, SmemLines<V>{sm, M},
+                run_plan_staged<typename F::plan, +1>(typename F::plan::seq{}, tw, lines, map, sx, ContigTile<V, F>{sm},
                                                       dst);
                 return;
             }
@@ -629,7 +641,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
         // the first pass
         constexpr bool kStage = sizeof(V) == 16;
         constexpr int kRow = 128 / (int)sizeof(V);
-        V *xs = sm + (lines * M + kRow - 1) / kRow * kRow;
+        V *xs = sm + contig_tile_elems(lines * M, kRow, F::plan::pad);
         if constexpr (kStage) {
             const V *xin = in + b0 * ld;
             const int per = M + 1;
@@ -656,11 +668,11 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
                 DfFlags bad;
                 const C2RPre<V, dcx> sdf{xsrc, (const dcx *)d.post_df, M, xld, valid, &bad};
                 const GlobalLinesOut<V, dcx> ddf{reinterpret_cast<V *>(out) + b0 * M, M, valid, dfl(scale)};
-                const SmemLines<dcx> tdf{reinterpret_cast<dcx *>(sm), M};
+                const ContigTile<dcx, F> tdf{reinterpret_cast<dcx *>(sm)};
                 if (df_stage<typename F::plan, +1, false>((const dcx *)d.twdf, lines, map, sdf, tdf, ddf, bad)) return;
             }
         }
-        const SmemLines<V> tile{sm, M};
+        const ContigTile<V, F> tile{sm};
         const C2RPre<V> sx{xsrc, post_tw, M, xld, valid};
         run_plan<typename F::plan, +1, false, F::split>(tw, lines, map, sx, tile, dst, d.mma);
     }
@@ -730,30 +742,31 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
     X(160, 16, 5, 2) X(192, 16, 4, 3) X(256, 16, 16) X(384, 16, 8, 3) X(512, 16, 16, 2)             \
     X(1024, 16, 16, 4) X(2048, 16, 16, 8) X(4096, 16, 16, 16)
 
-// The other 2/3/5-smooth lengths up to 1024 (3, 5, 6, 9, ... 1000): radix sequences as
-// radix_sequence() picks them, the fewest passes first.  A line of the generic kernels costs one
+// The other 2/3/5-smooth lengths up to 1024 (3, 5, 6, 9, ... 1000): as few passes as
+// radices up to 16 allow, in the order with the fewest bank conflicts in a contiguous tile (an odd
+// radix first where there is one, see SmemTile).  A line of the generic kernels costs one
 // shared-memory round trip per pass plus two to stage the tile, with run-time lengths in every
 // index and one tile per CTA in flight.  Measured, generic kernels -> these: a c2c stage of 243^3
 // complex64 304-367 -> 66-75 us (230 MB through HBM: 34 us), the N1 stage of 320 x 300 x 500 r2c
-// 393 -> 91 us, its r2c stage 469 -> 147 us; complex128 (bound by the FP64 pipe) 250 -> 186-232 us
+// 393 -> 91 us, its r2c stage 469 -> 100 us; complex128 (bound by the FP64 pipe) 250 -> 186-232 us
 // a stage of 180 x 200 x 216 r2c, from fewer inter-pass twiddles.
 // Above 1024 points lines are rare enough to stay with the generic kernels.  (Four groups: one
 // translation unit each per precision.)
 #define AFFT_SMOOTH_PLANS_A(X)                                                                      \
-    X(18, 6, 3) X(20, 5, 4) X(36, 6, 6) X(81, 9, 9) X(90, 10, 9) X(200, 8, 5, 5) X(243, 9, 9, 3)    \
-    X(250, 10, 5, 5) X(320, 8, 8, 5) X(450, 10, 9, 5) X(500, 10, 10, 5) X(625, 5, 5, 5, 5)          \
-    X(640, 10, 8, 8) X(675, 15, 9, 5) X(750, 15, 10, 5) X(810, 10, 9, 9)
+    X(18, 3, 6) X(20, 5, 4) X(36, 9, 4) X(81, 9, 9) X(90, 10, 9) X(200, 5, 5, 8) X(243, 9, 3, 9)    \
+    X(250, 5, 5, 10) X(320, 5, 8, 8) X(450, 9, 5, 10) X(500, 10, 5, 10) X(625, 5, 5, 5, 5)          \
+    X(640, 8, 8, 10) X(675, 15, 5, 9) X(750, 15, 5, 10) X(810, 10, 9, 9)
 #define AFFT_SMOOTH_PLANS_B(X)                                                                      \
-    X(6, 6) X(9, 9) X(27, 9, 3) X(30, 6, 5) X(72, 9, 8) X(125, 5, 5, 5) X(135, 15, 9)               \
-    X(180, 15, 12) X(216, 6, 6, 6) X(240, 16, 15) X(270, 9, 6, 5) X(432, 9, 8, 6)                   \
-    X(480, 10, 8, 6) X(540, 10, 9, 6) X(729, 9, 9, 9) X(864, 12, 9, 8) X(960, 12, 10, 8)
+    X(6, 6) X(9, 9) X(27, 9, 3) X(30, 5, 6) X(72, 9, 8) X(125, 5, 5, 5) X(135, 15, 9)               \
+    X(180, 15, 12) X(216, 6, 9, 4) X(240, 16, 15) X(270, 6, 9, 5) X(432, 6, 9, 8)                   \
+    X(480, 8, 6, 10) X(540, 6, 9, 10) X(729, 9, 9, 9) X(864, 9, 8, 12) X(960, 8, 10, 12)
 #define AFFT_SMOOTH_PLANS_C(X)                                                                      \
-    X(3, 3) X(12, 12) X(25, 5, 5) X(45, 9, 5) X(50, 10, 5) X(75, 15, 5) X(108, 12, 9)               \
-    X(225, 15, 15) X(288, 8, 6, 6) X(324, 9, 6, 6) X(360, 9, 8, 5) X(400, 10, 8, 5)                 \
-    X(486, 9, 9, 6) X(648, 9, 9, 8) X(720, 10, 9, 8) X(900, 10, 10, 9) X(972, 12, 9, 9)
+    X(3, 3) X(12, 12) X(25, 5, 5) X(45, 9, 5) X(50, 10, 5) X(75, 15, 5) X(108, 9, 12)               \
+    X(225, 15, 15) X(288, 8, 6, 6) X(324, 6, 9, 6) X(360, 9, 5, 8) X(400, 5, 8, 10)                 \
+    X(486, 6, 9, 9) X(648, 9, 8, 9) X(720, 9, 8, 10) X(900, 10, 9, 10) X(972, 9, 9, 12)
 #define AFFT_SMOOTH_PLANS_D(X)                                                                      \
-    X(5, 5) X(10, 10) X(15, 15) X(40, 8, 5) X(54, 9, 6) X(100, 10, 10) X(144, 12, 12)               \
-    X(150, 15, 10) X(162, 9, 6, 3) X(300, 10, 6, 5) X(375, 15, 5, 5) X(405, 9, 9, 5)                \
-    X(576, 9, 8, 8) X(600, 10, 10, 6) X(768, 12, 8, 8) X(800, 10, 10, 8) X(1000, 10, 10, 10)
+    X(5, 5) X(10, 10) X(15, 15) X(40, 8, 5) X(54, 9, 6) X(100, 10, 10) X(144, 16, 9)                \
+    X(150, 15, 10) X(162, 6, 9, 3) X(300, 5, 6, 10) X(375, 15, 5, 5) X(405, 9, 5, 9)                \
+    X(576, 9, 8, 8) X(600, 6, 10, 10) X(768, 8, 8, 12) X(800, 8, 10, 10) X(1000, 10, 10, 10)
 
 }  // namespace afft

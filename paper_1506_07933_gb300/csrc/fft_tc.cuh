@@ -215,9 +215,9 @@ __device__ __forceinline__ void tc16_pass(int n, int Ns, const float2 *__restric
 #pragma unroll
         for (int r = 0; r < 16; ++r) x[r] = src(l, j + r * nb);
         if (Ns > 1) {
-            const float2 *w = tw + (j % Ns) * 15;
+            const float2 *w = tw + j % Ns;
 #pragma unroll
-            for (int r = 1; r < 16; ++r) x[r] = ctw<S>(x[r], tw_ld<TwSmem>(w + r - 1));
+            for (int r = 1; r < 16; ++r) x[r] = ctw<S>(x[r], tw_ld<TwSmem>(w + (r - 1) * Ns));
         }
         float m = 0.f;
 #pragma unroll

@@ -154,7 +154,7 @@ bool shape_contig(Axis &a, long long nlines, size_t elem, size_t max_smem, bool 
     const int row = (int)(128 / elem);
     for (;;) {
         const int thr = threads_for(a.d, lines);
-        const size_t smem = ((size_t)lines * a.d.n + row - 1) / row * row * elem;
+        const size_t smem = (size_t)contig_tile_elems(lines * a.d.n, row, a.ks->contig_pad) * elem;
         if (thr <= a.ks->max_threads && smem <= max_smem) {
             a.lines = lines;
             a.log2_lines = 0;
@@ -195,8 +195,8 @@ __global__ void k_noalloc_twiddles(V *tw, const __grid_constant__ TwJob job)
         int s = 0;
         while (s + 1 < job.nseg && i >= job.base[s + 1]) ++s;
         const int local = i - job.base[s];
-        const int k = local / (job.R[s] - 1);
-        const int r = local - k * (job.R[s] - 1) + 1;
+        const int r = local / job.Ns[s] + 1;
+        const int k = local - (r - 1) * job.Ns[s];
         L = job.R[s] * job.Ns[s];
         m = (int)(((long long)r * k) % L);
     }
