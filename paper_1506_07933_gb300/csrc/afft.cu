@@ -453,13 +453,14 @@ int plan_shapes(afft_plan *p)
                       cudaFuncSetAttribute(ks->pipe_rp_early[k], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            ks->pipe_smem_rp) == cudaSuccess);
             int rs = 0;
-            if (ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rs, ks->pipe_rp[0], ks->pipe_threads,
+            if (ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&rs, ks->pipe_rp[0], ks->pipe_threads_rp,
                                                                     ks->pipe_smem_rp) == cudaSuccess && rs >= 1)
                 ap.rp_slots = sms * rs;
-            // early release by default when the first pass works on column pairs (radix <= 8):
-            // measured on 512-point N1 stages 0.207 -> 0.201 ms, while a radix-16 first pass
-            // (384 = 16 x 8 x 3) measured 0.100 -> 0.112 ms; the autotuner tries both
-            ap.rp_early = ap.rp_slots > 0 && ks->pipe_rp_early[0] && ks->radix[0] <= 8;
+            // early release by default when every pass works on column pairs (radix <= 8): measured
+            // on 512-point N1 stages 0.202 -> 0.197 ms, while single-column passes lost (120 = 8 x 15
+            // 39 -> 53 us, 256 = 16 x 16 0.201 -> 0.216 ms, 384 = 16 x 8 x 3 0.100 -> 0.115 ms); the
+            // autotuner tries both
+            ap.rp_early = ap.rp_slots > 0 && ks->pipe_rp_early[0] && ks->rp_all_pairs;
             cudaGetLastError();
         }
     }
@@ -673,7 +674,7 @@ cudaError_t strided_pipe(const AxisPlan &a, const V *in, V *out, const V *tw, lo
                         (void *)&tpo, (void *)&nt,  (void *)&err, (void *)&twdf, (void *)&mma, (void *)&rev};
         const void *fn = a.rp_early && a.ks->pipe_rp_early[0] ? a.ks->pipe_rp_early[backward ? 1 : 0]
                                                               : a.ks->pipe_rp[backward ? 1 : 0];
-        return cudaLaunchKernel(fn, dim3(grid), dim3(a.ks->pipe_threads), args, (size_t)a.ks->pipe_smem_rp, s);
+        return cudaLaunchKernel(fn, dim3(grid), dim3(a.ks->pipe_threads_rp), args, (size_t)a.ks->pipe_smem_rp, s);
     }
     const bool tma = encode_strided_map(&map, in, outer, a.desc.n, W, sizeof(V), a.ks->pipe_lines);
     if (!tma && !a.ks->pipe[PIPE_FWD_CPASYNC]) return cudaErrorNotSupported;

@@ -184,10 +184,12 @@ struct KernelSet {
     int pipe_smem;                 // its dynamic shared memory (two tile buffers)
     // complex64 families: the pipelined kernels for rows of odd width, read as row pairs
     // through TMA ([0] forward, [1] backward; the first ten arguments of pipe[], see
-    // k_strided_pipe_rp) and their shared memory; null / 0 elsewhere
+    // k_strided_pipe_rp), their shared memory and CTA size; null / 0 elsewhere
     const void *pipe_rp[2];
     const void *pipe_rp_early[2];  // the same with the load buffer released after the first pass
     int pipe_smem_rp;
+    int pipe_threads_rp;
+    bool rp_all_pairs;             // every row-pair pass works on column pairs (radices <= 8)
 };
 
 // Specialised kernels for line length n, or nullptr.

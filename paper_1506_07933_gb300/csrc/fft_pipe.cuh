@@ -61,12 +61,16 @@ template <typename V, int LG> struct SmemRowsC {
     __device__ __forceinline__ void operator()(int l, int p, V v) const { sm[(p << LG) + l] = v; }
 };
 
-template <int LG> struct MapLineFastC {
+template <int LG, bool Define = true> struct MapLineFastC {
     __device__ __forceinline__ void operator()(int idx, int, int &l, int &j) const
     {
         l = idx & ((1 << LG) - 1);
         j = idx >> LG;
     }
+};
+
+template <int LG, bool Define, typename V> struct DefineBoth<MapLineFastC<LG, Define>, V> {
+    static constexpr bool value = Define;
 };
 
 // ------------------------------------------------------------------ shape ---
@@ -80,7 +84,7 @@ template <int LG> struct MapLineFastC {
 // carries at most 16 complex values per pass.
 constexpr int kPipeSmemCap = 200 * 1024;
 
-template <class P, typename V> struct PipeShape {
+template <class P, typename V, int PairValues = 16, bool RowPairs = false> struct PipeShape {
     static constexpr int row_lines = 128 / (int)sizeof(V);
     __host__ __device__ static constexpr int lines_for(int l)
     {
@@ -88,21 +92,19 @@ template <class P, typename V> struct PipeShape {
     }
     static constexpr int lines = lines_for(row_lines);
     static constexpr int lg = lines == 16 ? 4 : lines == 8 ? 3 : lines == 4 ? 2 : lines == 2 ? 1 : 0;
-    __host__ __device__ static constexpr bool pairs(int r) { return sizeof(V) == 8 && lines >= 2 && 2 * r <= 16; }
+    __host__ __device__ static constexpr bool pairs(int r) { return sizeof(V) == 8 && lines >= 2 && 2 * r <= PairValues; }
     template <int... Rs> __host__ __device__ static constexpr int max_radix(Seq<Rs...>)
     {
         int m = 1;
         for (int r : {Rs...}) m = r > m ? r : m;
         return m;
     }
-    template <int R0, int... Rs> __host__ __device__ static constexpr int first_radix(Seq<R0, Rs...>) { return R0; }
-    static constexpr bool first_pairs = pairs(first_radix(typename P::seq{}));
     // butterflies (or butterfly pairs) per thread; complex128 tiles (float-float arithmetic, twice
     // the registers per value) of plans without a radix-16 pass carry at most 8 values per thread,
     // for more warps per SM
     __host__ __device__ static constexpr int per_thread(int r)
     {
-        return pairs(r) ? (16 / (2 * r) > 0 ? 16 / (2 * r) : 1)
+        return pairs(r) ? (PairValues / (2 * r) > 0 ? PairValues / (2 * r) : 1)
                : (sizeof(V) == 16 && P::df && max_radix(typename P::seq{}) <= 8) ? (8 / r > 1 ? 8 / r : 1)
                                                                       : bmax_for_radix(r);
     }
@@ -121,6 +123,30 @@ template <class P, typename V> struct PipeShape {
     // butterflies (or pairs) per thread that cover a radix-r pass with `threads` threads: in-place
     // passes hold all of them in registers across the barrier, so no more than needed
     __host__ __device__ static constexpr int covering(int r) { return (units(r) + threads - 1) / threads; }
+    // every pass' butterflies fill the CTA exactly / every pass works on column pairs
+    template <int... Rs> __host__ __device__ static constexpr bool exact_for(Seq<Rs...>)
+    {
+        bool e = true;
+        for (int r : {Rs...}) e = e && units(r) == threads * covering(r);
+        return e;
+    }
+    template <int... Rs> __host__ __device__ static constexpr bool pairs_for(Seq<Rs...>)
+    {
+        bool e = true;
+        for (int r : {Rs...}) e = e && pairs(r);
+        return e;
+    }
+    static constexpr bool all_pairs = pairs_for(typename P::seq{});
+    template <int... Rs> __host__ __device__ static constexpr bool singles_for(Seq<Rs...>)
+    {
+        bool e = true;
+        for (int r : {Rs...}) e = e && !pairs(r);
+        return e;
+    }
+    // thread map of the single-column passes (DefineBoth; row-pair tiles with only such passes, all
+    // of them exact -- 256 points -- measured faster without: 194 against 200 us on N1 of 8 x 256^3,
+    // while 128 = 16 x 8 gains: 101 -> 93 us on N1 of 32 x 128^3)
+    using map = MapLineFastC<lg, !(RowPairs && exact_for(typename P::seq{}) && singles_for(typename P::seq{}))>;
     using seq = typename P::seq;
     static constexpr int npass = P::npass;
     static constexpr int tile = P::n * lines;                       // complex elements per tile
@@ -155,17 +181,20 @@ template <class P, typename V> struct PipeShape {
     // CTAs per SM the launch bounds ask for: two when two such CTAs' shared memory fits (tiles,
     // table and the tensor-core state, about 5 KB of static shared memory)
     static constexpr int min_blocks_split = 2 * (smem + 6 * 1024) <= 226 * 1024 ? 2 : 1;
-    // smooth lengths: as many CTAs as the tiles leave room for, at 64 registers a thread (a
-    // radix-16 butterfly of complex64) or 128 (complex128)
+    // smooth lengths: as many CTAs as the tiles leave room for, at 64 registers a thread (16
+    // complex64 values, 80 for 20) or 128 (complex128)
     __host__ __device__ static constexpr int blocks_for(int bytes)
     {
-        const int by_smem = 226 * 1024 / (bytes + 1024), by_regs = 65536 / (threads * (sizeof(V) == 8 ? 64 : 128));
+        const int by_smem = 226 * 1024 / (bytes + 1024), by_regs = 65536 / (threads * (sizeof(V) == 8 ? 4 * PairValues : 128));
         const int b = by_smem < by_regs ? by_smem : by_regs;
         return b < 1 ? 1 : (b > 4 ? 4 : b);
     }
     static constexpr int min_blocks = P::smooth ? blocks_for(smem) : 1;
     static constexpr int min_blocks_rp = P::smooth ? blocks_for(smem_rp) : 1;
 };
+
+// Row-pair tiles (k_strided_pipe_rp) carry at most 16 values per thread at every length.
+template <class P> using RpShape = PipeShape<P, float2, 16, true>;
 
 // ---------------------------------------------------------- pair passes ---
 
@@ -284,21 +313,21 @@ __device__ __forceinline__ void pipe_passes(Seq<R, Rest...>, V *X, V *C, const V
         const SmemRowsC<V, LG> in_rows{src};
         constexpr int B = Sh::per_thread(R);
         if constexpr (Last && Split && R == 16)
-            spec_pass<R, S, false, Split, NT, B, TC, TwSmem>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, in_rows,
+            spec_pass<R, S, false, Split, NT, B, TC, TwSmem>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, in_rows,
                                                              out.cols, mma, src);
         else if constexpr (Split && R == 16)
-            spec_pass<R, S, false, Split, NT, B, TC, TwSmem>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, in_rows,
+            spec_pass<R, S, false, Split, NT, B, TC, TwSmem>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, in_rows,
                                                              SmemRowsC<V, LG>{dst}, mma, src);
         else if constexpr (Last && TwSmem)
-            radix_pass<R, S, false, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, in_rows, out.single);
+            radix_pass<R, S, false, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, in_rows, out.single);
         else if constexpr (TwSmem)
-            radix_pass<R, S, false, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, in_rows,
+            radix_pass<R, S, false, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, in_rows,
                                                  SmemRowsC<V, LG>{dst});
         else if constexpr (Last)
-            spec_pass<R, S, false, Split, NT, B>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, in_rows,
+            spec_pass<R, S, false, Split, NT, B>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, in_rows,
                                                  out.single, mma);
         else
-            spec_pass<R, S, false, Split, NT, B>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, in_rows,
+            spec_pass<R, S, false, Split, NT, B>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, in_rows,
                                                  SmemRowsC<V, LG>{dst}, mma);
     }
     if constexpr (!Last) {
@@ -322,8 +351,8 @@ __device__ __forceinline__ void scratch_passes(Seq<R, Rest...>, float2 *C, const
     } else {
         const SmemRowsC<float2, LG> rows{C};
         if constexpr (Global)
-            radix_pass<R, S, false, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, rows, out.single);
-        else radix_pass<R, S, true, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, MapLineFastC<LG>{}, rows, rows);
+            radix_pass<R, S, false, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, rows, out.single);
+        else radix_pass<R, S, true, NT, B, true>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{}, rows, rows);
     }
     if constexpr (sizeof...(Rest) > 0) {
         __syncthreads();
@@ -343,7 +372,7 @@ __device__ __forceinline__ void early_release_passes(Seq<R0, Rest...>, const flo
     if constexpr (Sh::pairs(R0))
         pair_pass<R0, S, N, 1, LG, NT, B>(X, tw, PairSmemOut<LG>{C});
     else
-        radix_pass<R0, S, false, NT, B>(N, 1, tw, Sh::lines, MapLineFastC<LG>{}, SmemRowsC<float2, LG>{const_cast<float2 *>(X)},
+        radix_pass<R0, S, false, NT, B>(N, 1, tw, Sh::lines, typename Sh::map{}, SmemRowsC<float2, LG>{const_cast<float2 *>(X)},
                                         SmemRowsC<float2, LG>{C});
     __syncthreads();
     released();
@@ -360,7 +389,7 @@ __device__ __forceinline__ bool pipe_df(Seq<R0, Rest...>, double2 *X, double2 *C
     constexpr int LG = Sh::lg, NT = Sh::threads;
     DfFlags bad;
     const SmemRowsConvIn<double2, dcx, LG> src{X, &bad};
-    radix_pass<R0, S, false, NT, Sh::per_thread(R0)>(N, 1, tw, Sh::lines, MapLineFastC<LG>{}, src,
+    radix_pass<R0, S, false, NT, Sh::per_thread(R0)>(N, 1, tw, Sh::lines, typename Sh::map{}, src,
                                  SmemRowsC<dcx, LG>{reinterpret_cast<dcx *>(C)});
     if (!df_tile_ok(bad)) return false;
     pipe_passes<Sh, S, N, R0, 0, 1>(Seq<Rest...>{}, reinterpret_cast<dcx *>(X), reinterpret_cast<dcx *>(C), tw, out);
@@ -601,9 +630,9 @@ __device__ __forceinline__ void rp_passes(Seq<R0, Rest...>, float2 *X, float2 *C
         constexpr int B = Sh::per_thread(R0);
         const RowPairIn<LW> in{A, Bx, l};
         if constexpr (Last)
-            radix_pass<R0, S, false, NT, B>(N, 1, tw, Sh::lines, MapLineFastC<LG>{}, in, out.single);
+            radix_pass<R0, S, false, NT, B>(N, 1, tw, Sh::lines, typename Sh::map{}, in, out.single);
         else
-            radix_pass<R0, S, false, NT, B>(N, 1, tw, Sh::lines, MapLineFastC<LG>{}, in, SmemRowsC<float2, LG>{C});
+            radix_pass<R0, S, false, NT, B>(N, 1, tw, Sh::lines, typename Sh::map{}, in, SmemRowsC<float2, LG>{C});
     }
     if constexpr (!Last) {
         __syncthreads();
@@ -624,7 +653,7 @@ __device__ __forceinline__ void rp_early_passes(Seq<R0, Rest...>, const float2 *
     if constexpr (Sh::pairs(R0))
         pair_pass_rp<R0, S, N, LW, LG, NT, Sh::per_thread(R0)>(A, Bx, PairSmemOut<LG>{C});
     else
-        radix_pass<R0, S, false, NT, Sh::per_thread(R0)>(N, 1, tw, Sh::lines, MapLineFastC<LG>{}, RowPairIn<LW>{A, Bx, l},
+        radix_pass<R0, S, false, NT, Sh::per_thread(R0)>(N, 1, tw, Sh::lines, typename Sh::map{}, RowPairIn<LW>{A, Bx, l},
                                                         SmemRowsC<float2, LG>{C});
     __syncthreads();
     released();
@@ -636,13 +665,13 @@ __device__ __forceinline__ void rp_early_passes(Seq<R0, Rest...>, const float2 *
 // of 18 x n/2).  Early: the load buffer is released after the first pass
 // (two tile loads in flight during the other passes), as k_strided_pipe does.
 template <class P, int S, bool Early = false>
-__global__ void __launch_bounds__(PipeShape<P, float2>::threads, PipeShape<P, float2>::min_blocks_rp)
+__global__ void __launch_bounds__(RpShape<P>::threads, RpShape<P>::min_blocks_rp)
     k_strided_pipe_rp(const float2 *__restrict__, float2 *out, const __grid_constant__ CUtensorMap tmap,
                       const float2 *__restrict__ tw, long long W, long long tiles_per_outer, long long ntiles,
                       unsigned *err, const void *, const unsigned *, int rev)
 {
     using V = float2;
-    using Sh = PipeShape<P, V>;
+    using Sh = RpShape<P>;
     constexpr int N = P::n, LINES = Sh::lines, LW = Sh::lw, TILE_RP = Sh::tile_rp;
     constexpr unsigned BOX_BYTES = (N / 2) * LW * sizeof(V);
     static_assert(Sh::rp_ok, "row-pair tiles: 16 complex64 columns, n even, at most 512");
@@ -878,8 +907,8 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, 1)
     }
 }
 
-// The kernels of one family as untyped entry points for the host.
-template <class F, typename V> KernelSet kernel_set(int n, int npass, const int *radix)
+// The kernels of one family as untyped entry points for the host (Contig: with the contiguous ones).
+template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, int npass, const int *radix)
 {
     KernelSet k{};
     k.n = n;
@@ -887,10 +916,12 @@ template <class F, typename V> KernelSet kernel_set(int n, int npass, const int 
     for (int i = 0; i < npass && i < kMaxPasses; ++i) k.radix[i] = radix[i];
     k.fn[KS_STRIDED_FWD] = (const void *)k_strided<F, -1, V>;
     k.fn[KS_STRIDED_BWD] = (const void *)k_strided<F, +1, V>;
-    k.fn[KS_CONTIG_FWD] = (const void *)k_contig<F, -1, V>;
-    k.fn[KS_CONTIG_BWD] = (const void *)k_contig<F, +1, V>;
-    k.fn[KS_R2C] = (const void *)k_r2c<F, V>;
-    k.fn[KS_C2R] = (const void *)k_c2r<F, V>;
+    if constexpr (Contig) {
+        k.fn[KS_CONTIG_FWD] = (const void *)k_contig<F, -1, V>;
+        k.fn[KS_CONTIG_BWD] = (const void *)k_contig<F, +1, V>;
+        k.fn[KS_R2C] = (const void *)k_r2c<F, V>;
+        k.fn[KS_C2R] = (const void *)k_c2r<F, V>;
+    }
     k.max_threads = F::template threads<V>();
     k.generic = F::generic;
     k.contig_pad = F::plan::pad;
@@ -904,7 +935,7 @@ template <class F, typename V> KernelSet kernel_set(int n, int npass, const int 
         // single-buffered kernel with the same rows, so it keeps the non-pipelined kernel.
         if constexpr (F::plan::smooth) {
             // TMA tiles alone (rows that no tensor map covers take k_strided), one row-pair form
-            // (early release when the first pass works on column pairs), no blocked layout and no
+            // (early release when every pass works on column pairs), no blocked layout and no
             // fused Poisson operator: what the generic kernels served before had none of these
             using P = typename F::plan;
             using Sh = PipeShape<P, V>;
@@ -915,7 +946,8 @@ template <class F, typename V> KernelSet kernel_set(int n, int npass, const int 
                 k.pipe_threads = Sh::threads;
                 k.pipe_smem = Sh::smem;
                 if constexpr (Sh::rp_ok) {
-                    constexpr bool early = P::npass >= 2 && Sh::first_pairs;
+                    constexpr bool early = P::npass >= 2 && RpShape<P>::all_pairs;
+                    k.pipe_threads_rp = RpShape<P>::threads;
                     k.pipe_rp[0] = (const void *)k_strided_pipe_rp<P, -1, early>;
                     k.pipe_rp[1] = (const void *)k_strided_pipe_rp<P, +1, early>;
                     k.pipe_smem_rp = Sh::smem_rp;
@@ -939,6 +971,8 @@ template <class F, typename V> KernelSet kernel_set(int n, int npass, const int 
             k.pipe_threads = Sh::threads;
             k.pipe_smem = Sh::smem;
             if constexpr (Sh::rp_ok && !F::split) {
+                k.pipe_threads_rp = RpShape<P>::threads;
+                k.rp_all_pairs = RpShape<P>::all_pairs;
                 k.pipe_rp[0] = (const void *)k_strided_pipe_rp<P, -1>;
                 k.pipe_rp[1] = (const void *)k_strided_pipe_rp<P, +1>;
                 if constexpr (P::npass >= 2) {

@@ -25,7 +25,10 @@
 // item or poll.
 //
 // The tile bodies are those of the specialised stage kernels (compile-time
-// radix sequences, complex64), instantiated for a fixed set of line lengths.
+// radix sequences, complex64), inlined into one kernel per direction for a
+// fixed set of line lengths.  (As called functions they took generic pointers and
+// kept 200 to 700 bytes each on the stack: 12.9 ms for the round trip of the
+// 200-field workload, 7.95 ms inlined at the same tile size.)
 #pragma once
 
 #include "fft_stage.cuh"
@@ -36,8 +39,13 @@ namespace afft {
 enum : unsigned char { QOP_R2C = 0, QOP_Y_FWD, QOP_X_FWD, QOP_X_BWD, QOP_Y_BWD, QOP_C2R };
 constexpr unsigned kQNone = 0xffffffffu;
 constexpr int kQMaxGroups = 8;
-constexpr int kQThreads = 512;
-constexpr int kQPoints = 8192;               // complex points per tile (64 KB of complex64)
+// Tiles of 4096 points on 256-thread CTAs, four per SM: a CTA waits on its counter, its loads and
+// its barriers in turn, so the number of CTAs is what hides them.  Measured on the 200-field
+// workload, round trip: 8192 points, 512 threads, two CTAs per SM 7.95 ms; 4096 points, 256 threads,
+// three 7.90 ms, four 7.14 ms.
+constexpr int kQThreads = 256;
+constexpr int kQBlocks = 4;
+constexpr int kQPoints = 4096;               // complex points per tile (32 KB of complex64)
 
 // Columns per strided tile for lines of n points: about kQPoints / n, a power of two from
 // 16 (128-byte rows) to 64 (the same on host and device).
@@ -75,8 +83,14 @@ struct QParams {
 
 // --------------------------------------------------------------- bodies ---
 
+// The bodies' thread maps (passes in the item loop define their values, see DefineBoth).
+struct QMapButterflyFast : MapButterflyFast {};
+struct QMapLineFast : MapLineFast {};
+template <typename V> struct DefineBoth<QMapButterflyFast, V> { static constexpr bool value = true; };
+template <typename V> struct DefineBoth<QMapLineFast, V> { static constexpr bool value = true; };
+
 template <class P>
-__device__ __noinline__ void q_r2c(const QGroup &g, unsigned plane, unsigned k, float2 *sm)
+__device__ __forceinline__ void q_r2c(const QGroup &g, unsigned plane, unsigned k, float2 *sm)
 {
     constexpr int M = P::n;
     const long long b0 = (long long)plane * g.n1 + (long long)k * g.zlines;
@@ -84,7 +98,7 @@ __device__ __noinline__ void q_r2c(const QGroup &g, unsigned plane, unsigned k, 
     // the input is the caller's array, written before the launch: plain loads
     const GlobalLines<float2> src{reinterpret_cast<const float2 *>(g.in) + b0 * M, M, valid};
     const SmemTile<float2, M, P::pad> tile{sm};
-    run_plan<P, -1, true>(g.tw[2], g.zlines, MapButterflyFast{}, src, tile, tile);
+    run_plan<P, -1, true>(g.tw[2], g.zlines, QMapButterflyFast{}, src, tile, tile);
     __syncthreads();
     float2 *o = reinterpret_cast<float2 *>(g.out) + b0 * (M + 1);
     if (!r2c_post_fixed_k<M, float2, float2>(tile, o, g.post, M + 1, valid))
@@ -92,7 +106,7 @@ __device__ __noinline__ void q_r2c(const QGroup &g, unsigned plane, unsigned k, 
 }
 
 template <class P, int S>
-__device__ __noinline__ void q_strided(const float2 *in, float2 *out, const float2 *tw, long long W,
+__device__ __forceinline__ void q_strided(const float2 *in, float2 *out, const float2 *tw, long long W,
                                           long long o, unsigned tile, float2 *sm)
 {
     constexpr int N = P::n, LINES = q_lines_for(P::n), LG = q_log2(LINES);
@@ -101,11 +115,11 @@ __device__ __noinline__ void q_strided(const float2 *in, float2 *out, const floa
     const int valid = (int)min((long long)LINES, W - c0);
     const GlobalCols<float2, float2, true> src{in + off, W, valid};
     const GlobalColsOut<float2> dst{out + off, W, valid};
-    run_plan<P, S, false>(tw, LINES, MapLineFast{LG}, src, SmemRows<float2>{sm, LG}, dst);
+    run_plan<P, S, false>(tw, LINES, QMapLineFast{{LG}}, src, SmemRows<float2>{sm, LG}, dst);
 }
 
 template <class P>
-__device__ __noinline__ void q_c2r(const QGroup &g, unsigned plane, unsigned k, float2 *sm)
+__device__ __forceinline__ void q_c2r(const QGroup &g, unsigned plane, unsigned k, float2 *sm)
 {
     constexpr int M = P::n;
     const long long b0 = (long long)plane * g.n1 + (long long)k * g.zlines;
@@ -124,11 +138,11 @@ __device__ __noinline__ void q_c2r(const QGroup &g, unsigned plane, unsigned k, 
         cp_async_wait<0>();
         __syncthreads();
         const C2RPre<float2> sx{sm, g.post, M, M + 1, valid};
-        run_plan_staged<P, +1>(typename P::seq{}, g.tw[2], g.zlines, MapButterflyFast{}, sx,
+        run_plan_staged<P, +1>(typename P::seq{}, g.tw[2], g.zlines, QMapButterflyFast{}, sx,
                                SmemTile<float2, M, P::pad>{sm}, dst);
     } else {
         const C2RPre<float2, float2, true> sx{xin, g.post, M, M + 1, valid};
-        run_plan<P, +1, false>(g.tw[2], g.zlines, MapButterflyFast{}, sx, SmemTile<float2, M, P::pad>{sm}, dst);
+        run_plan<P, +1, false>(g.tw[2], g.zlines, QMapButterflyFast{}, sx, SmemTile<float2, M, P::pad>{sm}, dst);
     }
 }
 
@@ -154,36 +168,25 @@ template <int S> struct QStrided {
     template <class P> __device__ __forceinline__ void run() const { q_strided<P, S>(in, out, tw, W, o, tile, sm); }
 };
 
-template <class... Ps> __device__ __forceinline__ void q_run_half(QFams<Ps...>, int op, int fam, const QGroup &g,
-                                                                 unsigned a, unsigned b, float2 *sm)
+template <bool Backward, class... Ps>
+__device__ __forceinline__ void q_run_half(QFams<Ps...>, int fam, const QGroup &g, unsigned a, unsigned b, float2 *sm)
 {
-    if (op == QOP_R2C) q_dispatch<QR2C, Ps...>(fam, QR2C{g, a, b, sm});
-    else q_dispatch<QC2R, Ps...>(fam, QC2R{g, a, b, sm});
+    if constexpr (Backward) q_dispatch<QC2R, Ps...>(fam, QC2R{g, a, b, sm});
+    else q_dispatch<QR2C, Ps...>(fam, QR2C{g, a, b, sm});
 }
 
-template <class... Ps> __device__ __forceinline__ void q_run_strided(QFams<Ps...>, int op, int fam, const QGroup &g,
-                                                                    unsigned a, unsigned b, float2 *sm)
+// A strided tile: N1 or N0, in place on the forward output or the backward workspace; the backward
+// N0 stage reads the input spectrum (which is never modified).
+template <bool Backward, class... Ps>
+__device__ __forceinline__ void q_run_strided(QFams<Ps...>, int op, int fam, const QGroup &g, unsigned a, unsigned b,
+                                              float2 *sm)
 {
-    const long long W1 = g.nh, W0 = (long long)g.n1 * g.nh;
-    switch (op) {
-    case QOP_Y_FWD: {   // in place on the forward output
-        float2 *x = reinterpret_cast<float2 *>(g.out);
-        q_dispatch<QStrided<-1>, Ps...>(fam, QStrided<-1>{x, x, g.tw[1], W1, a, b, sm});
-        break;
-    }
-    case QOP_X_FWD: {
-        float2 *x = reinterpret_cast<float2 *>(g.out);
-        q_dispatch<QStrided<-1>, Ps...>(fam, QStrided<-1>{x, x, g.tw[0], W0, a, b, sm});
-        break;
-    }
-    case QOP_X_BWD:     // input spectrum -> workspace (the input is never modified)
-        q_dispatch<QStrided<+1>, Ps...>(fam, QStrided<+1>{reinterpret_cast<const float2 *>(g.in), g.work,
-                                                          g.tw[0], W0, a, b, sm});
-        break;
-    default:            // QOP_Y_BWD, in place on the workspace
-        q_dispatch<QStrided<+1>, Ps...>(fam, QStrided<+1>{g.work, g.work, g.tw[1], W1, a, b, sm});
-        break;
-    }
+    const bool n0 = op == QOP_X_FWD || op == QOP_X_BWD;
+    float2 *x = Backward ? g.work : reinterpret_cast<float2 *>(g.out);
+    const float2 *in = Backward && n0 ? reinterpret_cast<const float2 *>(g.in) : x;
+    const long long W = n0 ? (long long)g.n1 * g.nh : g.nh;
+    constexpr int S = Backward ? +1 : -1;
+    q_dispatch<QStrided<S>, Ps...>(fam, QStrided<S>{in, x, n0 ? g.tw[0] : g.tw[1], W, a, b, sm});
 }
 
 // Relaxed load of a counter (device scope).
@@ -204,8 +207,8 @@ __device__ __forceinline__ unsigned long long q_now()
 // The persistent executor: Half lists the r2c/c2r families (half lengths M),
 // Full the strided families (n0, n1).  err: set on a wait that ran out;
 // abort: tells every CTA to stop.
-template <class Half, class Full>
-__global__ void __launch_bounds__(kQThreads, 2)
+template <class Half, class Full, bool Backward>
+__global__ void __launch_bounds__(kQThreads, kQBlocks)
     k_queue(const __grid_constant__ QParams prm, const QItem *__restrict__ items, unsigned nitems,
             unsigned *counters, unsigned *err, unsigned *abort_flag)
 {
@@ -246,8 +249,8 @@ __global__ void __launch_bounds__(kQThreads, 2)
             pre = w != kQNone ? q_load(counters + w) : 0;
         }
         const QGroup &g = prm.g[it.group];
-        if (it.op == QOP_R2C || it.op == QOP_C2R) q_run_half(Half{}, it.op, it.fam, g, it.a, it.b, sm);
-        else q_run_strided(Full{}, it.op, it.fam, g, it.a, it.b, sm);
+        if (it.op == (Backward ? QOP_C2R : QOP_R2C)) q_run_half<Backward>(Half{}, it.fam, g, it.a, it.b, sm);
+        else q_run_strided<Backward>(Full{}, it.op, it.fam, g, it.a, it.b, sm);
         __syncthreads();   // every thread's stores are issued, every shared read is done
         if (threadIdx.x == 0 && it.signal != kQNone) {
             __threadfence();   // release side: the CTA's stores before the increment

@@ -53,6 +53,15 @@ struct MapButterflyFast {  // contiguous stage: consecutive threads walk along a
     }
 };
 
+// Whether a pass defines its values on both sides of `this thread has a butterfly`.  Left undefined
+// on the idle side, they are live around the tile loop of a persistent kernel (that side carries
+// the last tile's): 20 to 60 registers, and spills where those are short.  The persistent strided
+// kernels and the multi-plan executor define them (complex128 512^3 r2c N1/N0 1137/1105 ->
+// 1041/1014 us, 192 points 156/148 -> 131/122 us); in one-tile kernels, and in the column-pair passes
+// of complex64 tiles (pair_pass), whose registers suffice, the second branch only costs (r2c lines
+// of 320 x 300 x 500 100 -> 118 us, N0 stage of 16 x 160^3 87 -> 90 us).
+template <class Map, typename V> struct DefineBoth { static constexpr bool value = false; };
+
 // ------------------------------------------------------ one radix pass ------
 // Thread t handles butterflies idx = t, t + blockDim.x, ... (at most
 // bmax_for_radix(R) of them; the host sizes the CTA so that suffices).  With
@@ -75,7 +84,7 @@ __device__ __forceinline__ void radix_pass(int n, int Ns, const V *__restrict__ 
         const int idx = threadIdx.x + b * nthr;
         lb[b] = -1;
         jb[b] = 0;
-        if (idx < total) {
+        if ((DefineBoth<Map, V>::value && NT > 0 && B * NT == total) || idx < total) {
             int l, j;
             map(idx, nb, l, j);
             lb[b] = l;
@@ -88,6 +97,9 @@ __device__ __forceinline__ void radix_pass(int n, int Ns, const V *__restrict__ 
                 for (int r = 1; r < R; ++r) v[b][r] = ctw<S>(v[b][r], tw_ld<TwSmem>(t + (r - 1) * Ns));
             }
             Dft<R, S, V>::run(v[b]);
+        } else if constexpr (DefineBoth<Map, V>::value) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[b][r] = czero<V>();
         }
     }
     if (InPlace) __syncthreads();

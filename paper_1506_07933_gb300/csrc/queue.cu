@@ -37,9 +37,12 @@ constexpr int kFullN[] = {48, 64, 96, 120, 128, 160, 256};
 const int kHalfR[][4] = {{8, 3}, {8, 4}, {16, 3}, {4, 3, 5}, {8, 8}, {16, 5}, {16, 8}};
 const int kFullR[][4] = {{16, 3}, {8, 8}, {8, 4, 3}, {8, 3, 5}, {16, 8}, {8, 4, 5}, {16, 16}};
 
-const void *queue_kernel() { return (const void *)k_queue<QHalf, QFull>; }
+const void *queue_kernel(int backward)
+{
+    return backward ? (const void *)k_queue<QHalf, QFull, true> : (const void *)k_queue<QHalf, QFull, false>;
+}
 
-constexpr size_t kQSmem = 72 * 1024;   // the largest tile: 8192 complex64 points, or c2r staging
+constexpr size_t kQSmem = (size_t)kQPoints * 9;   // the largest tile, padded, or its c2r staging
 
 int family(const int *ns, const int (*rad)[4], int count, const PlanView &v, int axis)
 {
@@ -208,7 +211,7 @@ struct afft_queue {
     unsigned nitems[2] = {0, 0};
     unsigned *d_counters = nullptr;   // counters, then the error flag, then the abort flag
     unsigned ncounters = 0;
-    int grid = 0;
+    int grid[2] = {0, 0};
     int device = 0;
 };
 
@@ -254,19 +257,24 @@ int afft_queue_create(afft_queue **out, int nplans, afft_plan *const *plans)
         q->groups.push_back(g);
     }
     q->ncounters = nc;
-    int per_sm = 0, sms = 0;
+    int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, q->device);
     int st = AFFT_OK;
-    if (cudaFuncSetAttribute(queue_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQSmem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, queue_kernel(), kQThreads, kQSmem) != cudaSuccess ||
-        per_sm < 1)
-        st = AFFT_ERR_CUDA;
-    q->grid = sms * per_sm;
+    for (int dir = 0; dir < 2 && st == AFFT_OK; ++dir) {
+        int per_sm = 0;
+        if (cudaFuncSetAttribute(queue_kernel(dir), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQSmem) !=
+                cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, queue_kernel(dir), kQThreads, kQSmem) !=
+                cudaSuccess ||
+            per_sm < 1)
+            st = AFFT_ERR_CUDA;
+        q->grid[dir] = sms * per_sm;
+    }
     for (int dir = 0; dir < 2 && st == AFFT_OK; ++dir) {
         // a dependency emitted two rounds of the grid earlier has usually finished; fields begun
         // but not finished are kept to 96 MB (of the 126 MB L2).  Measured on the 200-field
         // workload, forward: one round and 48 MB 8.1 ms, two rounds and 96 MB 6.6 ms
-        const std::vector<QItem> items = order_items(q->groups, dir == 1, nc, 2 * q->grid, 96.0 * (1 << 20));
+        const std::vector<QItem> items = order_items(q->groups, dir == 1, nc, 2 * q->grid[dir], 96.0 * (1 << 20));
         q->nitems[dir] = (unsigned)items.size();
         if (cudaMalloc(&q->d_items[dir], items.size() * sizeof(QItem)) != cudaSuccess) {
             q->d_items[dir] = nullptr;
@@ -326,9 +334,9 @@ int afft_queue_execute(afft_queue *q, int backward, const void *const *in, void 
     unsigned n = q->nitems[dir];
     unsigned *counters = q->d_counters, *err = q->d_counters + q->ncounters, *abort_flag = err + 1;
     void *args[] = {(void *)&prm, (void *)&items, (void *)&n, (void *)&counters, (void *)&err, (void *)&abort_flag};
-    const unsigned grid = (unsigned)std::min<long long>(q->grid, n);
+    const unsigned grid = (unsigned)std::min<long long>(q->grid[dir], n);
     if (grid == 0) return AFFT_OK;
-    return cudaLaunchKernel(queue_kernel(), dim3(grid), dim3(kQThreads), args, kQSmem, s) == cudaSuccess
+    return cudaLaunchKernel(queue_kernel(dir), dim3(grid), dim3(kQThreads), args, kQSmem, s) == cudaSuccess
                ? AFFT_OK
                : AFFT_ERR_CUDA;
 }
