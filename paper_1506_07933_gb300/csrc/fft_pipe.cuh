@@ -81,10 +81,14 @@ template <int LG, bool Define, typename V> struct DefineBoth<MapLineFastC<LG, De
 // kPipeSmemCap.  FP32 passes of radix <= 8 give each thread two adjacent
 // columns ("pairs": 16-byte shared-memory and global accesses, one twiddle
 // load for both); other passes give each thread one column.  Every thread
-// carries at most 16 complex values per pass.
+// carries at most 16 complex values per pass, 20 (PairValues) in the single-row
+// tiles of the smooth lengths, so that their radix-9 and radix-10 passes run as
+// pairs too: measured on N0 stages, 16 -> 20 values, 360 points (360 x 400 x 250
+// r2c, 4 fields) 241 -> 214 us, 600 points (600 x 720 x 500 c2c) 1197 -> 1096 us,
+// 320 points 77 -> 73 us; on row-pair tiles it lost (400 points 271 -> 297 us).
 constexpr int kPipeSmemCap = 200 * 1024;
 
-template <class P, typename V, int PairValues = 16, bool RowPairs = false> struct PipeShape {
+template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPairs = false> struct PipeShape {
     static constexpr int row_lines = 128 / (int)sizeof(V);
     __host__ __device__ static constexpr int lines_for(int l)
     {

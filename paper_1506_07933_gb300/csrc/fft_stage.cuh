@@ -739,16 +739,31 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
 // then the radices in pass order).  Split-precision plans use the sequences of
 // AFFT_SPLIT_LINE_PLANS (as many radix-16 passes as the length allows), and
 // the FP32 kernels for the other lengths of AFFT_LINE_PLANS (no radix-16 pass).
-// (Groups A-E only split the complex128 instantiations over translation units
-// that compile in parallel.)
-#define AFFT_LINE_PLANS_A(X)                                                                        \
-    X(1) X(2, 2) X(4, 4) X(8, 8) X(16, 16) X(24, 8, 3) X(32, 8, 4) X(48, 16, 3) X(60, 4, 3, 5) X(64, 8, 8)
-#define AFFT_LINE_PLANS_B(X) X(80, 16, 5) X(96, 8, 4, 3) X(120, 8, 3, 5) X(128, 16, 8) X(160, 8, 4, 5) X(192, 8, 8, 3)
-#define AFFT_LINE_PLANS_C(X) X(256, 16, 16) X(384, 16, 8, 3)
-#define AFFT_LINE_PLANS_D(X) X(512, 8, 8, 8) X(1024, 16, 8, 8)
-#define AFFT_LINE_PLANS_E(X) X(2048, 16, 16, 8) X(4096, 16, 16, 16)
+// The sequences are those that measured fastest over the strided and contiguous stages of cubes of
+// each length; complex128 (float-float, four registers per value) wants fewer values per thread, so
+// the two precisions differ.  Complex64, previous -> this: 60 = 4 3 5 -> 10 6 (c2c N2/N1/N0 of 64
+// fields 67/38/33 -> 45/35/31 us), 120 = 8 3 5 -> 8 15 (N1/N0 49/36 -> 40/34 us), 160 = 8 4 5 ->
+// 10 16 (121/90 -> 110/87 us), 192 = 8 8 3 -> 12 16 (94/79 -> 90/76 us, r2c of 384^3 102 -> 94 us).
+// Complex128: 384 = 16 8 3 -> 6 8 8 (611/578 -> 465/446 us, its fused Poisson stage 1879 -> 744 us:
+// radix 16 spills there), 1024 = 16 8 8 -> 8 8 4 4 (N1 of 64 x 1024^2 c2c 1213 -> 1126 us).  Measured
+// the same or slower: 128 = 8 4 4, 256 = 8 8 4, 384 = 6 8 8 and 1024 = 8 8 16 in complex64; 60 = 10 6,
+// 96 = 8 12, 120 = 8 15, 160 = 16 10 and 192 = 12 16 in complex128; 48 = 8 6 and 80 = 8 10 in either.
 #define AFFT_LINE_PLANS(X)                                                                          \
-    AFFT_LINE_PLANS_A(X) AFFT_LINE_PLANS_B(X) AFFT_LINE_PLANS_C(X) AFFT_LINE_PLANS_D(X) AFFT_LINE_PLANS_E(X)
+    X(1) X(2, 2) X(4, 4) X(8, 8) X(16, 16) X(24, 8, 3) X(32, 8, 4) X(48, 16, 3) X(60, 10, 6)        \
+    X(64, 8, 8) X(80, 16, 5) X(96, 8, 4, 3) X(120, 8, 15) X(128, 16, 8) X(160, 10, 16)              \
+    X(192, 12, 16) X(256, 16, 16) X(384, 16, 8, 3) X(512, 8, 8, 8) X(1024, 16, 8, 8)                \
+    X(2048, 16, 16, 8) X(4096, 16, 16, 16)
+// complex128, in five groups (the slowest instantiations to compile: one translation unit each)
+#define AFFT_LINE_PLANS_F64_A(X)                                                                    \
+    X(1) X(2, 2) X(4, 4) X(8, 8) X(16, 16) X(24, 8, 3) X(32, 8, 4) X(48, 16, 3) X(60, 4, 3, 5) X(64, 8, 8)
+#define AFFT_LINE_PLANS_F64_B(X) X(80, 16, 5) X(96, 8, 4, 3) X(120, 8, 3, 5) X(128, 16, 8) X(160, 8, 4, 5) X(192, 8, 8, 3)
+#define AFFT_LINE_PLANS_F64_C(X) X(256, 16, 16) X(384, 6, 8, 8)
+#define AFFT_LINE_PLANS_F64_D(X) X(512, 8, 8, 8) X(1024, 8, 8, 4, 4)
+#define AFFT_LINE_PLANS_F64_E(X) X(2048, 16, 16, 8) X(4096, 16, 16, 16)
+// complex128 lengths whose strided stages are faster with another sequence than their contiguous
+// ones (128 points: N1/N0 of 4 x 128^3 r2c 78/66 -> 66/62 us, but its r2c / c2r lines 172/183 ->
+// 172/192 us; 256 points: N1/N0 of 256^3 c2c 252/245 -> 234/235 us, its c2r lines 1345 -> 1413 us)
+#define AFFT_STRIDED_PLANS_F64(X) X(128, 8, 4, 4) X(256, 8, 8, 4)
 #define AFFT_SPLIT_LINE_PLANS(X)                                                                    \
     X(16, 16) X(32, 16, 2) X(48, 16, 3) X(64, 16, 4) X(80, 16, 5) X(96, 16, 3, 2) X(128, 16, 8)     \
     X(160, 16, 5, 2) X(192, 16, 4, 3) X(256, 16, 16) X(384, 16, 8, 3) X(512, 16, 16, 2)             \

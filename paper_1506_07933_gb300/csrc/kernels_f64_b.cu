@@ -1,5 +1,5 @@
 // kernels_f64_b.cu -- the double2 specialised families of the line lengths in
-// AFFT_LINE_PLANS_B (the complex128 instantiations are the slowest to compile,
+// AFFT_LINE_PLANS_F64_B (the complex128 instantiations are the slowest to compile,
 // so they are split over five translation units).
 #include "kernel_tables.cuh"
 
@@ -9,7 +9,7 @@ namespace afft {
 
 const KernelSet *spec_kernels_f64_b(int n)
 {
-    static const KernelSet table[] = {AFFT_LINE_PLANS_B(AFFT_X)};
+    static const KernelSet table[] = {AFFT_LINE_PLANS_F64_B(AFFT_X)};
     return find_set(table, n);
 }
 

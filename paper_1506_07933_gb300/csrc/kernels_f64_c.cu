@@ -1,5 +1,5 @@
 // kernels_f64_c.cu -- the double2 specialised families of the line lengths in
-// AFFT_LINE_PLANS_C (the complex128 instantiations are the slowest to compile,
+// AFFT_LINE_PLANS_F64_C (the complex128 instantiations are the slowest to compile,
 // so they are split over five translation units).
 #include "kernel_tables.cuh"
 
@@ -9,7 +9,7 @@ namespace afft {
 
 const KernelSet *spec_kernels_f64_c(int n)
 {
-    static const KernelSet table[] = {AFFT_LINE_PLANS_C(AFFT_X)};
+    static const KernelSet table[] = {AFFT_LINE_PLANS_F64_C(AFFT_X)};
     return find_set(table, n);
 }
 

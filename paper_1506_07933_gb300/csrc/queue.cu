@@ -28,14 +28,14 @@ namespace {
 
 // Families compiled into the executor: r2c/c2r half lengths and strided line lengths (the
 // radix sequences of the specialised kernels with the same length).
-using QHalf = QFams<LinePlan<24, 8, 3>, LinePlan<32, 8, 4>, LinePlan<48, 16, 3>, LinePlan<60, 4, 3, 5>,
+using QHalf = QFams<LinePlan<24, 8, 3>, LinePlan<32, 8, 4>, LinePlan<48, 16, 3>, LinePlan<60, 10, 6>,
                     LinePlan<64, 8, 8>, LinePlan<80, 16, 5>, LinePlan<128, 16, 8>>;
-using QFull = QFams<LinePlan<48, 16, 3>, LinePlan<64, 8, 8>, LinePlan<96, 8, 4, 3>, LinePlan<120, 8, 3, 5>,
-                    LinePlan<128, 16, 8>, LinePlan<160, 8, 4, 5>, LinePlan<256, 16, 16>>;
+using QFull = QFams<LinePlan<48, 16, 3>, LinePlan<64, 8, 8>, LinePlan<96, 8, 4, 3>, LinePlan<120, 8, 15>,
+                    LinePlan<128, 16, 8>, LinePlan<160, 10, 16>, LinePlan<256, 16, 16>>;
 constexpr int kHalfN[] = {24, 32, 48, 60, 64, 80, 128};
 constexpr int kFullN[] = {48, 64, 96, 120, 128, 160, 256};
-const int kHalfR[][4] = {{8, 3}, {8, 4}, {16, 3}, {4, 3, 5}, {8, 8}, {16, 5}, {16, 8}};
-const int kFullR[][4] = {{16, 3}, {8, 8}, {8, 4, 3}, {8, 3, 5}, {16, 8}, {8, 4, 5}, {16, 16}};
+const int kHalfR[][4] = {{8, 3}, {8, 4}, {16, 3}, {10, 6}, {8, 8}, {16, 5}, {16, 8}};
+const int kFullR[][4] = {{16, 3}, {8, 8}, {8, 4, 3}, {8, 15}, {16, 8}, {10, 16}, {16, 16}};
 
 const void *queue_kernel(int backward)
 {
