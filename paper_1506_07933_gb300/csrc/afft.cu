@@ -19,6 +19,7 @@
 
 #include "../../include/afft.h"
 #include "afft_internal.h"
+#include "fft_access.cuh"
 
 using namespace afft;
 
@@ -39,6 +40,7 @@ struct AxisPlan {
     int pipe_slots;        // CTAs resident at once (SMs x CTAs per SM): the persistent grid's cap
     int rp_slots;          // the same for the row-pair kernel of odd-width rows (0: none)
     bool rp_early;         // row-pair tiles release their load buffer after the first pass (tunable)
+    bool overlap;          // launched with programmatic dependent launch (launch_stage)
 };
 
 // Four-step split of one axis whose lines are longer than a CTA holds
@@ -247,6 +249,8 @@ bool shape_strided(const StageDesc &d, long long outer, long long W, size_t elem
     }
 }
 
+constexpr int kSMs = 152;   // GB300
+
 // Contiguous stage: whole lines, about `target` complex points per CTA
 // (0: 4096 for complex64, 2048 for complex128; the autotuner may pick others).
 // even_lines: an even count where possible, so that every CTA's run of lines of
@@ -255,7 +259,13 @@ bool shape_strided(const StageDesc &d, long long outer, long long W, size_t elem
 bool shape_contig(const StageDesc &d, const KernelSet *ks, long long nlines, size_t elem, size_t max_smem,
                   Launch &L, int target = 0, bool even_lines = false)
 {
-    if (target <= 0) target = elem == 8 ? 4096 : 2048;
+    if (target <= 0) {
+        target = elem == 8 ? 4096 : 2048;
+        // small complex64 arrays: down to one warp's worth of points per CTA, so that all SMs have
+        // work (the float-float kernels are bound by instruction fetch there and lose: 16 x 32 x 20 x
+        // 32 FP64 c2c 83 -> 98 us)
+        while (elem == 8 && target > 512 && nlines * d.n < 2LL * kSMs * target) target /= 2;
+    }
     int lines = std::max(1, target / std::max(1, d.n));
     lines = (int)std::min<long long>(lines, std::max(1LL, nlines));
     if (even_lines && lines > 1 && (lines & 1)) --lines;
@@ -270,6 +280,18 @@ bool shape_contig(const StageDesc &d, const KernelSet *ks, long long nlines, siz
             L.smem = smem;
             L.tiles_per_outer = 1;
             L.blocks = (nlines + lines - 1) / lines;
+            // twice the threads, half the butterflies each: for the c2r kernel of complex128 lines
+            // without a radix above 8 (its first pass is long: c2r of 384^3 643 -> 582 us, of 2 x 192^3
+            // 173 -> 156 us, while r2c and c2c lose, 618 -> 659 us), and for every kernel when the
+            // CTAs fill the chip at most twice, so that one butterfly's latency is what counts
+            // (128^3 r2c round trip 33 -> 31 us, 32^3 FP64 c2c 47 -> 34 us)
+            int rmax = 1;
+            for (int p = 0; p < d.npass; ++p) rmax = std::max(rmax, d.radix[p]);
+            L.c2r_threads = elem == 16 && !ks->generic && rmax <= 8 ? std::min(2 * thr, ks->max_threads) : thr;
+            if (!ks->generic && !ks->split && L.blocks <= 2 * kSMs) {
+                L.threads = std::min(2 * thr, ks->max_threads);
+                L.c2r_threads = std::max(L.c2r_threads, L.threads);
+            }
             return L.blocks > 0 && L.blocks < (1LL << 31);
         }
         if (lines == 1) return false;
@@ -530,11 +552,37 @@ size_t c2r_smem(const AxisPlan &a, size_t elem)
     return std::max(a.launch.smem, (staged + 127) / 128 * 128);
 }
 
+// Launches a stage kernel; with `overlap` its CTAs start while the previous kernel of the stream
+// finishes (programmatic dependent launch): they set up barriers and tables and wait in
+// stage_begin() for that kernel's completion, so the launch latency of each stage is hidden.
+// Complex64 plans of arrays up to kOverlapBytes use it: 64^3 Poisson solve 26.7 -> 18.9 us, 128^3 r2c
+// round trip 43.1 -> 33.0 us, 256^3 r2c 153 -> 144 us (135 MB).  Early CTAs land where the kernel that
+// is still running leaves room, not evenly: beyond L2 that costs more than the launch latency (32 x
+// 128^3 r2c, 540 MB, 563 -> 608 us; 1024^3 c2c 16.1 -> 25 ms), and in complex128, bound by arithmetic,
+// at every size (60 x 50 x 90 c2c 98 -> 172 us).  Not for split-precision plans either: a kernel that
+// waits while holding tensor memory could keep a CTA of its predecessor from allocating any.
+constexpr size_t kOverlapBytes = (size_t)144 << 20;
+cudaError_t launch_stage(const void *fn, long long blocks, int threads, void **args, size_t smem, cudaStream_t s,
+                         bool overlap)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 cudaError_t launch(const AxisPlan &a, int which, long long blocks, void **args, cudaStream_t s)
 {
     const Launch &L = a.launch;
     if (blocks <= 0) return cudaSuccess;
-    return cudaLaunchKernel(a.ks->fn[which], dim3((unsigned)blocks), dim3(L.threads), args, L.smem, s);
+    return launch_stage(a.ks->fn[which], blocks, L.threads, args, L.smem, s, a.overlap);
 }
 
 long long line_blocks(const AxisPlan &a, long long nlines)
@@ -654,7 +702,7 @@ cudaError_t pipe_on_map(const AxisPlan &a, const CUtensorMap &map, bool tma, con
     void *args[] = {(void *)&in,  (void *)&out, (void *)&map, (void *)&tw,   (void *)&W,
                     (void *)&tpo, (void *)&nt,  (void *)&err, (void *)&twdf, (void *)&mma, (void *)&rev};
     if (nt <= 0 || grid == 0) return nt <= 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
-    return cudaLaunchKernel(fn, dim3(grid), dim3(a.ks->pipe_threads), args, (size_t)a.ks->pipe_smem, s);
+    return launch_stage(fn, grid, a.ks->pipe_threads, args, (size_t)a.ks->pipe_smem, s, a.overlap);
 }
 
 // cudaErrorNotSupported, with nothing launched, when no kernel of the family loads these rows (the
@@ -678,7 +726,7 @@ cudaError_t strided_pipe(const AxisPlan &a, const V *in, V *out, const V *tw, lo
                         (void *)&tpo, (void *)&nt,  (void *)&err, (void *)&twdf, (void *)&mma, (void *)&rev};
         const void *fn = a.rp_early && a.ks->pipe_rp_early[0] ? a.ks->pipe_rp_early[backward ? 1 : 0]
                                                               : a.ks->pipe_rp[backward ? 1 : 0];
-        return cudaLaunchKernel(fn, dim3(grid), dim3(a.ks->pipe_threads_rp), args, (size_t)a.ks->pipe_smem_rp, s);
+        return launch_stage(fn, grid, a.ks->pipe_threads_rp, args, (size_t)a.ks->pipe_smem_rp, s, a.overlap);
     }
     const bool tma = encode_strided_map(&map, in, outer, a.desc.n, W, sizeof(V), a.ks->pipe_lines);
     if (!tma && !a.ks->pipe[PIPE_FWD_CPASYNC]) return cudaErrorNotSupported;
@@ -720,8 +768,8 @@ cudaError_t fourstep(const FourStep &f, const V *in, V *out, const V *tw, long l
                     (void *)&lg, (void *)&nb, (void *)&sc};
     const long long blocks = outer * f.nb * tpo;
     if (blocks <= 0) return cudaSuccess;
-    return cudaLaunchKernel(a.ks->four[backward ? 1 : 0], dim3((unsigned)blocks), dim3(a.launch.threads), args,
-                            a.launch.smem, s);
+    return launch_stage(a.ks->four[backward ? 1 : 0], blocks, a.launch.threads, args, a.launch.smem, s,
+                        a.overlap);
 }
 
 template <typename V>
@@ -763,8 +811,8 @@ cudaError_t c2r(const AxisPlan &a, const V *in, T *out, const V *tw, const V *po
                     (void *)&lines, (void *)&sc};
     const long long blocks = line_blocks(a, nlines);
     if (blocks <= 0) return cudaSuccess;
-    return cudaLaunchKernel(a.ks->fn[KS_C2R], dim3((unsigned)blocks), dim3(a.launch.threads), args,
-                            c2r_smem(a, sizeof(V)), s);
+    return launch_stage(a.ks->fn[KS_C2R], blocks, a.launch.c2r_threads, args, c2r_smem(a, sizeof(V)), s,
+                        a.overlap);
 }
 
 // Records the timing event `i` (0..3) of the current record, if timing is on.
@@ -898,6 +946,7 @@ template <typename V>
 __global__ void k_scale(V *x, long long count, double scale)
 {
     using T = decltype(V().x);
+    stage_begin();
     const T sc = (T)scale;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (long long)gridDim.x * blockDim.x) {
@@ -980,8 +1029,12 @@ int run_backward_axes(afft_plan *p, const void *in, void *out, cudaStream_t s)
             return AFFT_ERR_CUDA;
         if (p->bscale != 1.0) {
             const unsigned blocks = (unsigned)std::max<long long>(1, std::min<long long>((count + 255) / 256, 152LL * 16));
-            k_scale<V><<<blocks, 256, 0, s>>>((V *)out, count, p->bscale);
-            if (cudaGetLastError() != cudaSuccess) return AFFT_ERR_CUDA;
+            V *x = (V *)out;
+            long long n = count;
+            double sc = p->bscale;
+            void *args[] = {(void *)&x, (void *)&n, (void *)&sc};
+            if (launch_stage((const void *)k_scale<V>, blocks, 256, args, 0, s, p->ax[0].overlap) != cudaSuccess)
+                return AFFT_ERR_CUDA;
         }
     }
     mark(p, 3, s);
@@ -1173,8 +1226,8 @@ int run_poisson(afft_plan *p, const void *in, void *out, cudaStream_t s)
                         (void *)&tpo, (void *)&nt,   (void *)&err, (void *)&twdf,   (void *)&in1,
                         (void *)&ipitch, (void *)&inh, (void *)&rev};
         const unsigned grid = (unsigned)std::min<long long>(nt, x.pipe_slots);
-        if (cudaLaunchKernel(x.ks->poisson[tma ? 0 : 1], dim3(grid), dim3(x.ks->pipe_threads), args,
-                             (size_t)x.ks->pipe_smem, s) != cudaSuccess)
+        if (launch_stage(x.ks->poisson[tma ? 0 : 1], grid, x.ks->pipe_threads, args, (size_t)x.ks->pipe_smem, s,
+                         x.overlap) != cudaSuccess)
             return AFFT_ERR_CUDA;
     } else {
         if (n0 > 1 && axis_stage<V>(p, 0, w, w, B, W, 0, 1.0, s) != cudaSuccess) return AFFT_ERR_CUDA;
@@ -1184,7 +1237,8 @@ int run_poisson(afft_plan *p, const void *in, void *out, cudaStream_t s)
         void *args[] = {(void *)&w, (void *)&planes, (void *)&a0, (void *)&a1, (void *)&a2, (void *)&a3};
         const long long total = P0 * n1 * nh;
         const unsigned blocks = (unsigned)std::min<long long>((total + 255) / 256, 152LL * 32);
-        if (cudaLaunchKernel(g->poisson_mult, dim3(blocks), dim3(256), args, 0, s) != cudaSuccess) return AFFT_ERR_CUDA;
+        if (launch_stage(g->poisson_mult, blocks, 256, args, 0, s, x.overlap) != cudaSuccess)
+            return AFFT_ERR_CUDA;
         if (n0 > 1 && axis_stage<V>(p, 0, w, w, B, W, 1, 1.0, s) != cudaSuccess) return AFFT_ERR_CUDA;
     }
     mark(p, 2, s);
@@ -1343,6 +1397,10 @@ int afft_plan_create_axes(afft_plan **out, const int64_t n[3], int64_t batch, in
         delete p;
         return AFFT_ERR_CUDA;
     }
+
+    const bool overlap = precision == AFFT_F32 &&
+                         (double)batch * n[0] * n[1] * p->nh * cplx_size(precision) <= (double)kOverlapBytes;
+    for (int a = 0; a < 3; ++a) p->ax[a].overlap = p->four[a].a.overlap = overlap;
 
     std::vector<int> tm, tl;
     // an axis left untransformed gets the length-1 (copy) family, which its stage never launches

@@ -127,6 +127,7 @@ struct Launch {
     int lines;                     // lines (columns) per CTA
     int log2_lines;                // log2(lines) for the strided stage (lines is a power of 2)
     int threads;                   // threads per CTA
+    int c2r_threads;               // contiguous stage: threads per CTA of the c2r kernel
     size_t smem;                   // dynamic shared memory bytes
     long long blocks;              // grid size
     long long tiles_per_outer;     // strided stage: CTAs per outer slab
@@ -165,6 +166,7 @@ struct KernelSet {
     const void *fn[KS_COUNT];
     int max_threads;               // largest CTA the kernels were compiled for
     bool generic;
+    bool split;                    // radix-16 passes on the tensor cores
     bool contig_pad;               // the contiguous kernels pad their shared tile (contig_tile_elems)
     const void *pipe[PIPE_COUNT];  // null when the family has no pipelined strided kernel
     const void *pipe_blk[2];       // its blocked-row TMA variants ([0] forward, [1] backward)

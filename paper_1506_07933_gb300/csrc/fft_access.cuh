@@ -32,6 +32,16 @@ __device__ __forceinline__ void cp_async_zfill(void *dst, const void *src, bool 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
+// Start of a stage kernel (programmatic dependent launch, see launch_stage): lets the next
+// kernel of the stream launch as soon as every CTA of this one has started, then waits until the
+// previous kernel has finished and its writes are visible.  Only tables that no stage writes (the
+// twiddles) may be read before it.  Returns at once in a kernel launched without the attribute.
+__device__ __forceinline__ void stage_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // mbarriers (shared::cta) for the asynchronous copies of the tensor-memory
 // accelerator: initialisation, the expected byte count of a phase, and waits
 // bounded by %globaltimer.

@@ -436,6 +436,7 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, Split ? PipeShape<P,
         mbar_init(&bars[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    stage_begin();
     __syncthreads();
     // split precision: radix-16 passes on tcgen05 where the tile allows (fft_tc.cuh)
     constexpr bool TC = Split && sizeof(V) == 8;
@@ -709,6 +710,7 @@ __global__ void __launch_bounds__(RpShape<P>::threads, RpShape<P>::min_blocks_rp
         tma_load_3d(buf0 + b * TILE_RP + Sh::box_rp, &tmap, (int)(W + c0 - 1), 0, (int)o, &bars[b]);
     };
 
+    stage_begin();
     // Without Early the next tile's load is issued once this one has landed.
     issue(t, 0);
     if (Early && t + gridDim.x < ntiles) issue(t + gridDim.x, 1);
@@ -850,6 +852,7 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, 1)
         }
     };
 
+    stage_begin();
     // The load buffer is not released early here (unlike k_strided_pipe): the six passes of a
     // tile hide the next load already, and the in-place passes' extra barriers made the
     // 512-point operator slower.
@@ -928,6 +931,7 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
     }
     k.max_threads = F::template threads<V>();
     k.generic = F::generic;
+    k.split = F::split;
     k.contig_pad = F::plan::pad;
     if constexpr (F::generic) {
         k.four[0] = (const void *)k_fourstep<-1, V, F::split>;

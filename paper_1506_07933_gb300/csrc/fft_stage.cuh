@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
               const V *__restrict__ tw, long long W, long long tiles_per_outer, int log2_lines)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    stage_begin();
     V *sm = reinterpret_cast<V *>(smem_raw);
     const int n = F::generic ? d.n : F::plan::n;
     const int lines = 1 << log2_lines;
@@ -404,6 +405,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
              const V *__restrict__ tw, long long nlines, int lines, typename RealOf<V>::T scale)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    stage_begin();
     V *sm = reinterpret_cast<V *>(smem_raw);
     const int n = F::generic ? d.n : F::plan::n;
     const long long b0 = stage_order(blockIdx.x, gridDim.x, d.rev) * lines;
@@ -564,6 +566,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
 {
     using T = typename RealOf<V>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    stage_begin();
     V *sm = reinterpret_cast<V *>(smem_raw);
     const int M = F::generic ? d.n : F::plan::n;
     const long long b0 = stage_order(blockIdx.x, gridDim.x, d.rev) * lines;
@@ -614,6 +617,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
           typename RealOf<V>::T scale)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    stage_begin();
     V *sm = reinterpret_cast<V *>(smem_raw);
     const int M = F::generic ? d.n : F::plan::n;
     const long long b0 = stage_order(blockIdx.x, gridDim.x, d.rev) * lines;
@@ -701,6 +705,7 @@ __global__ void __launch_bounds__(256, 1)
                typename RealOf<V>::T scale)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    stage_begin();
     V *sm = reinterpret_cast<V *>(smem_raw);
     const int na = d.n;
     const int lines = 1 << log2_lines;
@@ -722,6 +727,7 @@ template <typename V>
 __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, int nh)
 {
     using T = typename RealOf<V>::T;
+    stage_begin();
     const long long total = planes * n1 * nhp;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
