@@ -34,6 +34,8 @@ struct AxisPlan {
     Launch launch;
     const KernelSet *ks;   // kernels for this line length (specialised or generic)
     int tw_base;           // first twiddle of this axis in the plan's table; desc.tw_off is relative
+    int twr_base;          // the same for the reversed radix sequence (axis 0 of r2c plans: Poisson solve)
+    int poisson_slots;     // CTAs of the fused Poisson kernel resident at once (0: the plan has none)
     // pipelined strided kernel (persistent CTAs) when the family has one
     bool pipe_avail;       // the family has it and it fits this device
     bool pipe;             // in use (the autotuner may switch it off)
@@ -173,22 +175,13 @@ const KernelSet *lookup_kernels(int precision, int64_t n, bool contiguous)
     return precision == AFFT_F64 ? generic_kernels_f64() : generic_kernels_f32();
 }
 
-// Fills desc for length n (with the radix sequence of the specialised kernel
-// when there is one) and appends its twiddle entries (m, L), meaning
-// exp(-2 pi i m / L), to the table lists.
-void build_desc(int64_t n, const KernelSet *ks, StageDesc &d, std::vector<int> &tm,
-                std::vector<int> &tl)
+// Fills desc for length n and the radix sequence `rad`, and appends its twiddle entries (m, L),
+// meaning exp(-2 pi i m / L), to the table lists.
+void build_desc(const std::vector<int> &rad, int64_t n, StageDesc &d, std::vector<int> &tm, std::vector<int> &tl)
 {
     std::memset(&d, 0, sizeof d);
     d.n = (int)n;
     const int base = (int)tm.size();
-    std::vector<int> rad;
-    if (!ks->generic) rad.assign(ks->radix, ks->radix + ks->npass);
-    else if (ks == generic_kernels_split()) rad = split_radix_plan(n);
-    else {
-        int r[kMaxPasses];
-        rad.assign(r, r + std::max(0, radix_sequence(n, r)));
-    }
     d.npass = (int)rad.size();
     int ns = 1;
     for (int p = 0; p < d.npass; ++p) {
@@ -206,6 +199,19 @@ void build_desc(int64_t n, const KernelSet *ks, StageDesc &d, std::vector<int> &
         }
         ns *= R;
     }
+}
+
+// The same with the radix sequence of the kernels (theirs when specialised).
+void build_desc(int64_t n, const KernelSet *ks, StageDesc &d, std::vector<int> &tm, std::vector<int> &tl)
+{
+    std::vector<int> rad;
+    if (!ks->generic) rad.assign(ks->radix, ks->radix + ks->npass);
+    else if (ks == generic_kernels_split()) rad = split_radix_plan(n);
+    else {
+        int r[kMaxPasses];
+        rad.assign(r, r + std::max(0, radix_sequence(n, r)));
+    }
+    build_desc(rad, n, d, tm, tl);
 }
 
 int required_threads(const StageDesc &d, int lines)
@@ -438,6 +444,7 @@ int plan_shapes(afft_plan *p)
         const KernelSet *ks = ap.ks;
         ap.pipe_avail = false;
         ap.pipe_slots = 0;
+        ap.poisson_slots = 0;
         if (ks->generic || !ks->pipe[PIPE_FWD_TMA] || ks->pipe_smem > max_smem) continue;
         for (int k = 0; k < PIPE_COUNT; ++k)
             if (ks->pipe[k] &&
@@ -449,8 +456,9 @@ int plan_shapes(afft_plan *p)
                                                         ks->pipe_smem) != cudaSuccess)
                 return AFFT_ERR_CUDA;
         for (int k = 0; k < 2; ++k)
-            if (ks->poisson[k] && cudaFuncSetAttribute(ks->poisson[k], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       ks->pipe_smem) != cudaSuccess)
+            if (ks->poisson[k] && ks->poisson_smem <= max_smem &&
+                cudaFuncSetAttribute(ks->poisson[k], cudaFuncAttributeMaxDynamicSharedMemorySize, ks->poisson_smem) !=
+                    cudaSuccess)
                 return AFFT_ERR_CUDA;
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ks->pipe[PIPE_FWD_TMA], ks->pipe_threads,
@@ -462,6 +470,11 @@ int plan_shapes(afft_plan *p)
             per_sm = std::max(per_sm, resident_per_sm(ks->pipe[PIPE_FWD_TMA], ks->pipe_threads, ks->pipe_smem,
                                                       p->device));
         if (per_sm < 1) continue;
+        int pois = 0;
+        if (ks->poisson[0] && ks->poisson_smem <= max_smem &&
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pois, ks->poisson[0], ks->pipe_threads, ks->poisson_smem) ==
+                cudaSuccess)
+            ap.poisson_slots = sms * pois;
         ap.pipe_slots = sms * per_sm;   // also what the blocked c2c layout runs with
         // rows far apart: the many CTAs of the plain kernel win in the row-major layout
         const bool far = ks->n >= 1024 && row_bytes[a] > (1LL << 22);
@@ -1211,22 +1224,25 @@ int run_poisson(afft_plan *p, const void *in, void *out, cudaStream_t s)
     mark(p, 1, s);
     const AxisPlan &x = p->ax[0];
     const long long W = n1 * nh;
-    if (n0 > 1 && x.pipe && !p->four[0].on && x.ks->poisson[0]) {
-        alignas(64) CUtensorMap map;
-        std::memset(&map, 0, sizeof map);
-        const bool tma = encode_strided_map(&map, w, B, x.desc.n, W, sizeof(V), x.ks->pipe_lines);
+    alignas(64) CUtensorMap map;
+    std::memset(&map, 0, sizeof map);
+    const bool fused = n0 > 1 && x.pipe && !p->four[0].on && x.poisson_slots > 0;
+    const bool tma = fused && encode_strided_map(&map, w, B, x.desc.n, W, sizeof(V), x.ks->pipe_lines);
+    if (fused && x.ks->poisson[tma ? 0 : 1]) {
         const V *twa = tw + x.tw_base;
         long long WW = W;
         long long tpo = (W + x.ks->pipe_lines - 1) / x.ks->pipe_lines, nt = B * tpo;
+        const V *twr = tw + x.twr_base;
         const void *twdf = x.desc.twdf;
+        const void *twrdf = p->d_twdf ? (const void *)((const char *)p->d_twdf + (size_t)x.twr_base * 16) : nullptr;
         unsigned *err = p->d_err;
         int in1 = (int)n1, ipitch = (int)nh, inh = (int)nh, rev = 0;
         const V *win = w;
         void *args[] = {(void *)&win, (void *)&w,    (void *)&map, (void *)&twa,    (void *)&WW,
                         (void *)&tpo, (void *)&nt,   (void *)&err, (void *)&twdf,   (void *)&in1,
-                        (void *)&ipitch, (void *)&inh, (void *)&rev};
-        const unsigned grid = (unsigned)std::min<long long>(nt, x.pipe_slots);
-        if (launch_stage(x.ks->poisson[tma ? 0 : 1], grid, x.ks->pipe_threads, args, (size_t)x.ks->pipe_smem, s,
+                        (void *)&ipitch, (void *)&inh, (void *)&rev, (void *)&twr, (void *)&twrdf};
+        const unsigned grid = (unsigned)std::min<long long>(nt, x.poisson_slots);
+        if (launch_stage(x.ks->poisson[tma ? 0 : 1], grid, x.ks->pipe_threads, args, (size_t)x.ks->poisson_smem, s,
                          x.overlap) != cudaSuccess)
             return AFFT_ERR_CUDA;
     } else {
@@ -1426,6 +1442,17 @@ int afft_plan_create_axes(afft_plan **out, const int64_t n[3], int64_t batch, in
                 tm.push_back((int)m);
                 tl.push_back((int)len[a]);
             }
+        }
+    }
+    p->ax[0].twr_base = p->ax[0].tw_base;
+    if (kind == AFFT_R2C && !p->four[0].on && p->ax[0].ks->poisson[0]) {
+        const StageDesc &d = p->ax[0].desc;
+        std::vector<int> back(d.radix, d.radix + d.npass);
+        std::reverse(back.begin(), back.end());
+        if (!std::equal(back.begin(), back.end(), d.radix)) {
+            p->ax[0].twr_base = (int)tm.size();
+            StageDesc unused;
+            build_desc(back, d.n, unused, tm, tl);
         }
     }
     p->post_off = (int)tm.size();

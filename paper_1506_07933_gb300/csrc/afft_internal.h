@@ -179,8 +179,10 @@ struct KernelSet {
     // fused Poisson N0 stage (forward DFTs, 1/|k|^2, inverse DFTs) on pipelined tiles:
     // (const V *in, V *out, CUtensorMap map, const V *tw, long long W,
     // long long tiles_per_outer, long long ntiles, unsigned *err, const void *twdf,
-    // int n1, int nhp, int nh, int rev); [0] TMA, [1] cp.async
+    // int n1, int nhp, int nh, int rev, const V *twr, const void *twrdf) (twr, twrdf: the twiddle
+    // tables of the reversed radix sequence); [0] TMA, [1] cp.async
     const void *poisson[2];
+    int poisson_smem;              // its dynamic shared memory
     int pipe_lines;                // columns per tile of the pipelined kernel
     int pipe_threads;              // its (compile-time) CTA size
     int pipe_smem;                 // its dynamic shared memory (two tile buffers)

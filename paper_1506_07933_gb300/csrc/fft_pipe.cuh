@@ -88,7 +88,8 @@ template <int LG, bool Define, typename V> struct DefineBoth<MapLineFastC<LG, De
 // 320 points 77 -> 73 us; on row-pair tiles it lost (400 points 271 -> 297 us).
 constexpr int kPipeSmemCap = 200 * 1024;
 
-template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPairs = false> struct PipeShape {
+template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPairs = false, bool DefinePairs = false> struct PipeShape {
+    static constexpr bool define_pairs = DefinePairs;   // pair passes define their values (DefineBoth)
     static constexpr int row_lines = 128 / (int)sizeof(V);
     __host__ __device__ static constexpr int lines_for(int l)
     {
@@ -141,6 +142,13 @@ template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPai
         return e;
     }
     static constexpr bool all_pairs = pairs_for(typename P::seq{});
+    template <int... Rs> __host__ __device__ static constexpr int last_radix(Seq<Rs...>)
+    {
+        int l = 0;
+        for (int r : {Rs...}) l = r;
+        return l;
+    }
+    static constexpr bool mid_pairs = pairs(last_radix(typename P::seq{}));   // the Poisson kernel's middle pass
     template <int... Rs> __host__ __device__ static constexpr bool singles_for(Seq<Rs...>)
     {
         bool e = true;
@@ -187,18 +195,24 @@ template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPai
     static constexpr int min_blocks_split = 2 * (smem + 6 * 1024) <= 226 * 1024 ? 2 : 1;
     // smooth lengths: as many CTAs as the tiles leave room for, at 64 registers a thread (16
     // complex64 values, 80 for 20) or 128 (complex128)
-    __host__ __device__ static constexpr int blocks_for(int bytes)
+    __host__ __device__ static constexpr int blocks_for(int bytes, int regs = sizeof(V) == 8 ? 4 * PairValues : 128)
     {
-        const int by_smem = 226 * 1024 / (bytes + 1024), by_regs = 65536 / (threads * (sizeof(V) == 8 ? 4 * PairValues : 128));
+        const int by_smem = 226 * 1024 / (bytes + 1024), by_regs = 65536 / (threads * regs);
         const int b = by_smem < by_regs ? by_smem : by_regs;
         return b < 1 ? 1 : (b > 4 ? 4 : b);
     }
     static constexpr int min_blocks = P::smooth ? blocks_for(smem) : 1;
+    // the fused Poisson kernel holds a second (reversed) twiddle table
+    static constexpr int twr_smem = tw_smem > 0 ? P::n - last_radix(seq{}) : 0;
+    static constexpr int smem_poisson = smem + twr_smem * 8;
+    static constexpr int min_blocks_poisson = blocks_for(smem_poisson, sizeof(V) == 8 || !P::df ? 128 : 168);
     static constexpr int min_blocks_rp = P::smooth ? blocks_for(smem_rp) : 1;
 };
 
 // Row-pair tiles (k_strided_pipe_rp) carry at most 16 values per thread at every length.
 template <class P> using RpShape = PipeShape<P, float2, 16, true>;
+// Fused Poisson tiles run twice the passes in one loop: their pair passes define their values.
+template <class P, typename V> using PoissonShape = PipeShape<P, V, P::smooth ? 20 : 16, false, true>;
 
 // ---------------------------------------------------------- pair passes ---
 
@@ -231,7 +245,8 @@ struct PairGlobalOut {
 // butterflies are (column pair lp, butterfly j), reading both columns' R
 // values with 16-byte loads and sharing the twiddles.  InPlace: every read of
 // the CTA precedes a barrier, every write follows it (src and dst may alias).
-template <int R, int S, int N, int Ns, int LG, int NT, int B, bool InPlace = false, bool TwSmem = false, class Dst>
+template <int R, int S, int N, int Ns, int LG, int NT, int B, bool InPlace = false, bool TwSmem = false,
+          bool Define = false, class Dst>
 __device__ __forceinline__ void pair_pass(const float2 *src, const float2 *__restrict__ tw, const Dst &dst)
 {
     constexpr int PAIRS = (1 << LG) / 2, NB = N / R, TOTAL = PAIRS * NB;
@@ -260,6 +275,9 @@ __device__ __forceinline__ void pair_pass(const float2 *src, const float2 *__res
             }
             Dft<R, S, float2>::run(lo[b]);
             Dft<R, S, float2>::run(hi[b]);
+        } else if constexpr (Define) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) lo[b][r] = hi[b][r] = make_float2(0.f, 0.f);
         }
     }
     if constexpr (InPlace) __syncthreads();
@@ -311,8 +329,10 @@ __device__ __forceinline__ void pipe_passes(Seq<R, Rest...>, V *X, V *C, const V
     V *dst = (Q % 2 == 0) ? C : X;
     if constexpr (Sh::pairs(R)) {
         constexpr int B = Sh::per_thread(R);
-        if constexpr (Last) pair_pass<R, S, N, Ns, LG, NT, B, false, TwSmem>(src, tw + TwOff, out.pair);
-        else pair_pass<R, S, N, Ns, LG, NT, B, false, TwSmem>(src, tw + TwOff, PairSmemOut<LG>{dst});
+        if constexpr (Last)
+            pair_pass<R, S, N, Ns, LG, NT, B, false, TwSmem, Sh::define_pairs>(src, tw + TwOff, out.pair);
+        else
+            pair_pass<R, S, N, Ns, LG, NT, B, false, TwSmem, Sh::define_pairs>(src, tw + TwOff, PairSmemOut<LG>{dst});
     } else {
         const SmemRowsC<V, LG> in_rows{src};
         constexpr int B = Sh::per_thread(R);
@@ -754,7 +774,12 @@ __global__ void __launch_bounds__(RpShape<P>::threads, RpShape<P>::min_blocks_rp
 // the r2c spectrum by |k|^2 (integer wavenumbers k_i = m for m <= n_i/2, else
 // m - n_i) and zeroes k = 0.  Its N0 stage is fused: forward N0 DFTs, the
 // division, inverse N0 DFTs, all on the tile in shared memory, so the
-// spectrum makes one HBM round trip instead of three.
+// spectrum makes one HBM round trip instead of three.  A tile of P passes runs
+// 2 P - 1 (the last forward pass, the division and the first inverse pass are one,
+// see poisson_mid): it is bound by shared memory and barriers, not by HBM.
+// Measured N0 operator, 2 P + 1 exchanges -> 2 P - 1: 8 x 256^3 FP32 332 -> 241 us (a plain N0 stage 181), 512^3
+// 369 -> 318 us, 32 x 128^3 139 -> 115 us, FP64 256^3 285 -> 238 us, 384^3 744 -> 699 us; the smooth lengths,
+// which ran three kernels: 320 x 300 x 500 249 -> 154 us.
 
 template <typename T> __device__ __forceinline__ T inv_int(int K);
 template <> __device__ __forceinline__ float inv_int<float>(int K) { return 1.0f / (float)K; }
@@ -766,48 +791,152 @@ template <> __device__ __forceinline__ dfl inv_int<dfl>(int K)
     return dfl(r, fmaf(-r, k, 1.0f) * r);
 }
 
-// Writes of the forward half's last pass into a shared tile (both pass kinds).
+// 1 / |k|^2 along one column: kk = k1^2 + k2^2 of the column, p = k0 (0 for the zero mode, and for
+// columns past the array's edge, keep = false).
+template <int N, typename V> struct PoissonColumn {
+    int kk;
+    bool keep;
+    __device__ __forceinline__ V operator()(V v, int p) const
+    {
+        using T = typename RealOf<V>::T;
+        const int k0w = 2 * p > N ? p - N : p;
+        const int K = k0w * k0w + kk;
+        return (keep && K > 0) ? cscale(v, inv_int<T>(K)) : czero<V>();
+    }
+};
+
+// The middle pass: the last forward pass of radix R leaves X[j + s N/R], s < R, in a thread's
+// registers, which are exactly the inputs j + r N/R of the first pass of an inverse transform that
+// starts with the same radix.  So the division and that inverse pass follow in registers, and the
+// inverse runs the radices in reverse order (its own twiddle table unless they are a palindrome).
+// src and dst differ, so each butterfly reads, computes and writes on its own.
+template <class Sh, int N, int R, bool TwSmem, typename V, class Dst>
+__device__ __forceinline__ void poisson_mid(const V *src, const V *__restrict__ tw, const Dst &dst,
+                                            const PoissonColumn<N, V> &c0, const PoissonColumn<N, V> &c1)
+{
+    constexpr int LG = Sh::lg, NT = Sh::threads, NB = N / R, TOTAL = Sh::units(R), B = Sh::covering(R);
+    if constexpr (Sh::pairs(R)) {
+        constexpr int PAIRS = (1 << LG) / 2;
+        const float4 *s4 = reinterpret_cast<const float4 *>(src);
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int idx = threadIdx.x + b * NT;
+            if (B * NT == TOTAL || idx < TOTAL) {
+                const int lp = idx % PAIRS, j = idx / PAIRS;
+                float2 lo[R], hi[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float4 q = s4[(j + r * NB) * PAIRS + lp];
+                    lo[r] = make_float2(q.x, q.y);
+                    hi[r] = make_float2(q.z, q.w);
+                    if (NB > 1 && r > 0) {
+                        const float2 w = tw_ld<TwSmem>(tw + j + (r - 1) * NB);
+                        lo[r] = ctw<-1>(lo[r], w);
+                        hi[r] = ctw<-1>(hi[r], w);
+                    }
+                }
+                Dft<R, -1, float2>::run(lo);
+                Dft<R, -1, float2>::run(hi);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    lo[r] = c0(lo[r], j + r * NB);
+                    hi[r] = c1(hi[r], j + r * NB);
+                }
+                Dft<R, +1, float2>::run(lo);
+                Dft<R, +1, float2>::run(hi);
+#pragma unroll
+                for (int r = 0; r < R; ++r) dst.pair(lp, j * R + r, lo[r], hi[r]);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int idx = threadIdx.x + b * NT;
+            if (B * NT == TOTAL || idx < TOTAL) {
+                const int l = idx & ((1 << LG) - 1), j = idx >> LG;
+                V v[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    v[r] = src[((j + r * NB) << LG) + l];
+                    if (NB > 1 && r > 0) v[r] = ctw<-1>(v[r], tw_ld<TwSmem>(tw + j + (r - 1) * NB));
+                }
+                Dft<R, -1, V>::run(v);
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r] = c0(cnorm(v[r]), j + r * NB);
+                Dft<R, +1, V>::run(v);
+#pragma unroll
+                for (int r = 0; r < R; ++r) dst.single(l, j * R + r, cnorm(v[r]));
+            }
+        }
+    }
+}
+
+// Output of the middle pass into a shared tile.
 template <typename V, int LG> struct SmemTileOut {
     SmemRowsC<V, LG> single;
     PairSmemOut<LG> pair;
 };
 
-// Forward N0 DFTs (tile A, scratch Bf), the 1/|k|^2 scaling, inverse N0 DFTs,
-// the last pass storing through `gout`.  The thread's column is fixed
-// (tid mod LINES), so its (k1, k2) are resolved once: col1 = k1, col2 = k2,
-// keep = false for pad columns.
-template <class Sh, int N, typename CT, class GOut>
-__device__ __forceinline__ void poisson_tile(CT *A, CT *Bf, const CT *tw, const GOut &gout, int n1, int k1,
-                                             int k2, bool keep)
+template <class Done, int... Rs> struct ReverseSeq;
+template <int... Ds> struct ReverseSeq<Seq<Ds...>> { using type = Seq<Ds...>; };
+template <int... Ds, int R, int... Rs> struct ReverseSeq<Seq<Ds...>, R, Rs...> : ReverseSeq<Seq<R, Ds...>, Rs...> {};
+
+// Forward passes Seq<R, Rest...> (Q: number of the first one; an even one reads X, an odd one C), the
+// middle pass, then the inverse passes Back (the radices before the middle one, reversed) with the
+// reversed table `twr`, the last one storing through `gout`.
+template <class Sh, int N, int Ns, int TwOff, int Q, bool TwSmem, typename V, class GOut, int... Back, int R, int... Rest>
+__device__ __forceinline__ void poisson_passes(Seq<R, Rest...>, Seq<Back...>, V *X, V *C, const V *tw, const V *twr,
+                                               const GOut &gout, const PoissonColumn<N, V> &c0,
+                                               const PoissonColumn<N, V> &c1)
 {
-    using T = typename RealOf<CT>::T;
-    constexpr int LG = Sh::lg, NT = Sh::threads, TILE = Sh::tile;
-    constexpr int NP = Sh::npass;
-    CT *D = (NP - 1) % 2 == 0 ? Bf : A;       // where the forward half's last pass writes
-    CT *E = D == Bf ? A : Bf;
-    SmemTileOut<CT, LG> mid;
-    mid.single = SmemRowsC<CT, LG>{D};
-    mid.pair = PairSmemOut<LG>{reinterpret_cast<float2 *>(D)};
-    pipe_passes<Sh, -1, N, 1, 0, 0>(typename Sh::seq{}, A, Bf, tw, mid);
-    __syncthreads();
-    const int k1w = 2 * k1 > n1 ? k1 - n1 : k1;
-    for (int e = threadIdx.x; e < TILE; e += NT) {
-        const int p = e >> LG;                 // k0 (natural order after the forward passes)
-        const int k0w = 2 * p > N ? p - N : p;
-        const int K = k0w * k0w + k1w * k1w + k2 * k2;
-        D[e] = (keep && K > 0) ? cscale(D[e], inv_int<T>(K)) : czero<CT>();
+    constexpr int LG = Sh::lg, NT = Sh::threads, B = Sh::per_thread(R);
+    V *src = (Q % 2 == 0) ? X : C, *dst = (Q % 2 == 0) ? C : X;
+    if constexpr (sizeof...(Rest) > 0) {
+        if constexpr (Sh::pairs(R))
+            pair_pass<R, -1, N, Ns, LG, NT, B, false, TwSmem, Sh::define_pairs>(src, tw + TwOff, PairSmemOut<LG>{dst});
+        else
+            radix_pass<R, -1, false, NT, B, TwSmem>(N, Ns, tw + TwOff, Sh::lines, typename Sh::map{},
+                                                    SmemRowsC<V, LG>{src}, SmemRowsC<V, LG>{dst});
+        __syncthreads();
+        poisson_passes<Sh, N, Ns * R, TwOff + (Ns > 1 ? Ns * (R - 1) : 0), Q + 1, TwSmem>(
+            Seq<Rest...>{}, Seq<R, Back...>{}, X, C, tw, twr, gout, c0, c1);
+    } else if constexpr (sizeof...(Back) == 0) {
+        poisson_mid<Sh, N, R, TwSmem>(src, tw + TwOff, gout, c0, c1);
+    } else {
+        SmemTileOut<V, LG> mid;
+        mid.single = SmemRowsC<V, LG>{dst};
+        mid.pair = PairSmemOut<LG>{reinterpret_cast<float2 *>(dst)};
+        poisson_mid<Sh, N, R, TwSmem>(src, tw + TwOff, mid, c0, c1);
+        __syncthreads();
+        pipe_passes<Sh, +1, N, R, 0, Q + 1, false, TwSmem>(Seq<Back...>{}, X, C, twr, gout);
     }
-    __syncthreads();
-    pipe_passes<Sh, +1, N, 1, 0, 0>(typename Sh::seq{}, D, E, tw, gout);
+}
+
+// FP64 tile in float-float: the first pass converts, as in pipe_df.  Returns false, with X
+// untouched, when some value was out of float-float range.
+template <class Sh, int N, class GOut, int R0, int... Rest>
+__device__ __forceinline__ bool poisson_df(Seq<R0, Rest...>, double2 *X, double2 *C, const dcx *tw, const dcx *twr,
+                                           const GOut &gout, const PoissonColumn<N, dcx> &c)
+{
+    constexpr int LG = Sh::lg;
+    DfFlags bad;
+    const SmemRowsConvIn<double2, dcx, LG> src{X, &bad};
+    radix_pass<R0, -1, false, Sh::threads, Sh::per_thread(R0)>(N, 1, tw, Sh::lines, typename Sh::map{}, src,
+                                                              SmemRowsC<dcx, LG>{reinterpret_cast<dcx *>(C)});
+    if (!df_tile_ok(bad)) return false;
+    poisson_passes<Sh, N, R0, 0, 1, false>(Seq<Rest...>{}, Seq<R0>{}, reinterpret_cast<dcx *>(X),
+                                           reinterpret_cast<dcx *>(C), tw, twr, gout, c, c);
+    return true;
 }
 
 template <class P, typename V, bool TMA>
-__global__ void __launch_bounds__(PipeShape<P, V>::threads, 1)
+__global__ void __launch_bounds__(PoissonShape<P, V>::threads, PoissonShape<P, V>::min_blocks_poisson)
     k_poisson_pipe(const V *__restrict__ in, V *out, const __grid_constant__ CUtensorMap tmap,
                    const V *__restrict__ tw, long long W, long long tiles_per_outer, long long ntiles,
-                   unsigned *err, const void *twdf, int n1, int nhp, int nh, int rev)
+                   unsigned *err, const void *twdf, int n1, int nhp, int nh, int rev,
+                   const V *__restrict__ twr, const void *twrdf)
 {
-    using Sh = PipeShape<P, V>;
+    using Sh = PoissonShape<P, V>;
     constexpr int N = P::n, LINES = Sh::lines, LG = Sh::lg, NT = Sh::threads, TILE = Sh::tile;
     constexpr unsigned TILE_BYTES = TILE * sizeof(V);
     extern __shared__ __align__(1024) unsigned char pipe_smem_raw[];
@@ -815,9 +944,16 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, 1)
     V *const scratch = buf0 + 2 * TILE;
     unsigned long long *const bars = reinterpret_cast<unsigned long long *>(pipe_smem_raw + 3 * TILE_BYTES);
     const int tid = threadIdx.x;
+    // complex64 tiles stage both twiddle tables (forward, reversed) behind the mbarriers
+    constexpr bool StageTw = sizeof(V) == 8;
+    V *const tw_s = reinterpret_cast<V *>(pipe_smem_raw + 3 * TILE_BYTES + 16);
 
     long long t = blockIdx.x;
     if (t >= ntiles) return;
+    if constexpr (StageTw) {
+        for (int e = tid; e < Sh::tw_smem; e += NT) tw_s[e] = ldgc(tw + e);
+        for (int e = tid; e < Sh::twr_smem; e += NT) tw_s[Sh::tw_smem + e] = ldgc(twr + e);
+    }
     if (TMA && tid == 0) {
         mbar_init(&bars[0], 1);
         mbar_init(&bars[1], 1);
@@ -853,9 +989,9 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, 1)
     };
 
     stage_begin();
-    // The load buffer is not released early here (unlike k_strided_pipe): the six passes of a
-    // tile hide the next load already, and the in-place passes' extra barriers made the
-    // 512-point operator slower.
+    // The load buffer is not released early here (unlike k_strided_pipe): the passes of a tile hide
+    // the next load already, and the in-place passes' extra barriers made the 512-point operator
+    // slower.
     issue(t, 0);
     for (int i = 0;; ++i) {
         const int b = i & 1;
@@ -875,29 +1011,34 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, 1)
         const long long tile = stage_order(t, ntiles, rev);
         const long long o = tile / tiles_per_outer;
         const long long c0 = (tile - o * tiles_per_outer) * LINES;
-        const long long c = c0 + (tid & (LINES - 1));
-        const int k1 = (int)(c / nhp), k2 = (int)(c - (long long)(c / nhp) * nhp);
-        const bool keep = c < W && k2 < nh;
         V *X = buf0 + b * TILE;
         V *obase = out + o * (long long)N * W;
+        auto kk_of = [&](long long c) {
+            const int k1 = (int)(c / nhp), k2 = (int)(c - (long long)k1 * nhp);
+            const int k1w = 2 * k1 > n1 ? k1 - n1 : k1;
+            return k1w * k1w + k2 * k2;
+        };
+        const long long c = c0 + (tid & (LINES - 1));
         bool done = false;
-        if constexpr (std::is_same<V, double2>::value) {
+        if constexpr (std::is_same<V, double2>::value && P::df) {
             if (twdf) {
-                // float-float: convert the tile into the scratch buffer, vote on range
-                DfFlags f;
-                dcx *Y = reinterpret_cast<dcx *>(scratch);
-                for (int e = tid; e < TILE; e += NT) Y[e] = Conv<dcx, double2>::in(X[e], &f);
-                if (df_tile_ok(f)) {
-                    TileOut<V, dcx> g;
-                    g.single = GlobalColFixedOut<V, dcx>{obase, W, c < W ? c : -1};
-                    poisson_tile<Sh, N>(Y, reinterpret_cast<dcx *>(X), (const dcx *)twdf, g, n1, k1, k2, keep);
-                    done = true;
-                }
+                TileOut<V, dcx> g;
+                g.single = GlobalColFixedOut<V, dcx>{obase, W, c < W ? c : -1};
+                const PoissonColumn<N, dcx> col{kk_of(c), c < W};
+                done = poisson_df<Sh, N>(typename Sh::seq{}, X, scratch, (const dcx *)twdf, (const dcx *)twrdf, g, col);
             }
         }
         if (!done) {
             TileOut<V> g;
             g.single = GlobalColFixedOut<V>{obase, W, c < W ? c : -1};
+            PoissonColumn<N, V> col0{}, col1{};
+            if constexpr (Sh::mid_pairs) {
+                const long long a = c0 + 2 * (tid % (LINES / 2));
+                col0 = PoissonColumn<N, V>{kk_of(a), a < W};
+                col1 = PoissonColumn<N, V>{kk_of(a + 1), a + 1 < W};
+            } else {
+                col0 = PoissonColumn<N, V>{kk_of(c), c < W};
+            }
             if constexpr (sizeof(V) == 8) {
                 const int lp = tid % (LINES / 2 > 0 ? LINES / 2 : 1);
                 const long long a = c0 + 2 * lp;
@@ -906,7 +1047,8 @@ __global__ void __launch_bounds__(PipeShape<P, V>::threads, 1)
                                  (reinterpret_cast<unsigned long long>(base) & 15) == 0;
                 g.pair = PairGlobalOut{base, W, a < W ? a : -1, a + 1 < W ? a + 1 : -1, vec};
             }
-            poisson_tile<Sh, N>(X, scratch, tw, g, n1, k1, k2, keep);
+            poisson_passes<Sh, N, 1, 0, 0, StageTw>(typename Sh::seq{}, Seq<>{}, X, scratch, StageTw ? tw_s : tw,
+                                                    StageTw ? tw_s + Sh::tw_smem : twr, g, col0, col1);
         }
         __syncthreads();   // the next tile's load into this buffer waits for every read
         if (tn >= ntiles) break;
@@ -943,8 +1085,7 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
         // single-buffered kernel with the same rows, so it keeps the non-pipelined kernel.
         if constexpr (F::plan::smooth) {
             // TMA tiles alone (rows that no tensor map covers take k_strided), one row-pair form
-            // (early release when every pass works on column pairs), no blocked layout and no
-            // fused Poisson operator: what the generic kernels served before had none of these
+            // (early release when every pass works on column pairs) and no blocked layout
             using P = typename F::plan;
             using Sh = PipeShape<P, V>;
             if constexpr (Sh::tma_ok) {
@@ -953,6 +1094,8 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
                 k.pipe_lines = Sh::lines;
                 k.pipe_threads = Sh::threads;
                 k.pipe_smem = Sh::smem;
+                k.poisson[0] = (const void *)k_poisson_pipe<P, V, true>;
+                k.poisson_smem = Sh::smem_poisson;
                 if constexpr (Sh::rp_ok) {
                     constexpr bool early = P::npass >= 2 && RpShape<P>::all_pairs;
                     k.pipe_threads_rp = RpShape<P>::threads;
@@ -974,6 +1117,7 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
             if constexpr (!F::split) {   // split plans run the Poisson multiply as its own kernel
                 k.poisson[0] = (const void *)k_poisson_pipe<P, V, true>;
                 k.poisson[1] = (const void *)k_poisson_pipe<P, V, false>;
+                k.poisson_smem = Sh::smem_poisson;
             }
             k.pipe_lines = Sh::lines;
             k.pipe_threads = Sh::threads;

@@ -91,3 +91,18 @@ def test_chained_launches_in_a_captured_graph(kind, prec):
         for i, (a, b) in enumerate(got):
             assert torch.equal(a, want[i % 3][0]) and torch.equal(b, want[i % 3][1]), i
     assert oracle.rel_l2(want[0][1].cpu().numpy(), xs[0].cpu().numpy()) <= (2e-6 if prec == "f32" else 1e-12)
+
+
+@pytest.mark.parametrize("n", [1] + sorted(MAIN | set(LENGTHS)))
+def test_poisson_every_n0_length(n):
+    """The fused N0 operator (forward, 1/|k|^2 and inverse in one middle pass) at every line length,
+    with a ragged last tile, and rows of odd width (which take the separate multiply)."""
+    for shape in ((n, 6, 12), (n, 5, 12)):
+        for prec in ("f32", "f64"):
+            f = synth.uniform_real(shape, n).astype(RDT[prec])
+            with afft.Plan(shape, "r2c", prec) as p:
+                u = p.poisson(torch.from_numpy(f).cuda())
+                torch.cuda.synchronize()
+                assert p.device_status() == 0
+            err = oracle.rel_l2(u.cpu().numpy(), oracle.poisson(f.astype(np.float64)))
+            assert err <= (2e-6 if prec == "f32" else 1e-12), (shape, prec, err)
