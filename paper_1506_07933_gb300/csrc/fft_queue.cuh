@@ -57,7 +57,7 @@ __host__ __device__ constexpr int q_lines_for(int n)
 }
 __host__ __device__ constexpr int q_log2(int v) { return v <= 1 ? 0 : 1 + q_log2(v / 2); }
 
-struct QItem {
+struct __align__(8) QItem {
     unsigned char op, group;
     unsigned short fam;                      // index into the executor's family list for this op
     unsigned a;                              // outer line (N1/N0/r2c/c2r: plane or field of the group)
@@ -215,19 +215,37 @@ __global__ void __launch_bounds__(kQThreads, kQBlocks)
     extern __shared__ __align__(128) unsigned char q_smem_raw[];
     float2 *sm = reinterpret_cast<float2 *>(q_smem_raw);
     __shared__ int s_go;
-    // thread 0 reads each item's counter one item ahead (relaxed), so that the round trip
-    // overlaps the previous item's work; the fence before the item makes it an acquire
-    unsigned pre = 0;
-    if (threadIdx.x == 0 && blockIdx.x < nitems && items[blockIdx.x].wait != kQNone)
-        pre = q_load(counters + items[blockIdx.x].wait);
-    for (unsigned i = blockIdx.x; i < nitems; i += gridDim.x) {
-        const QItem it = items[i];
+    // Thread 0 keeps the CTA's next two items in a ring of three (asynchronous copies, two items
+    // ahead) and reads the next item's counter and the abort flag during the current item, so that
+    // none of those L2 round trips stands between two items; the fence before the item makes the
+    // counter read an acquire.  Measured on the 200-field workload: 7.13 -> 7.00 ms.
+    __shared__ QItem s_item[3];
+    const unsigned G = gridDim.x;
+    auto fetch = [&](unsigned i, int slot) {
+        if (i < nitems) {
+            const char *g = reinterpret_cast<const char *>(items + i);
+            char *d = reinterpret_cast<char *>(&s_item[slot]);
+#pragma unroll
+            for (int k = 0; k < (int)sizeof(QItem); k += 8) cp_async_zfill<8>(d + k, g + k, true);
+        }
+        cp_async_commit();
+    };
+    unsigned pre = 0, aborted = 0;
+    if (threadIdx.x == 0) {
+        fetch(blockIdx.x, 0);
+        fetch(blockIdx.x + G, 1);
+        cp_async_wait<0>();
+        if (blockIdx.x < nitems && s_item[0].wait != kQNone) pre = q_load(counters + s_item[0].wait);
+    }
+    int slot = 0;
+    for (unsigned i = blockIdx.x; i < nitems; i += G) {
         if (threadIdx.x == 0) {
-            int go = q_load(abort_flag) == 0;
-            if (go && it.wait != kQNone && pre < it.need) {
+            const unsigned wait = s_item[slot].wait, need = s_item[slot].need;
+            int go = aborted == 0;
+            if (go && wait != kQNone && pre < need) {
                 const unsigned long long t0 = q_now();
                 for (unsigned k = 1;; ++k) {
-                    if (q_load(counters + it.wait) >= it.need) break;
+                    if (q_load(counters + wait) >= need) break;
                     if ((k & 63u) == 0) {
                         if (q_load(abort_flag) != 0) { go = 0; break; }
                         if (q_now() - t0 > 2000000000ull) {
@@ -242,20 +260,28 @@ __global__ void __launch_bounds__(kQThreads, kQBlocks)
             __threadfence();   // acquire side: the counter reads above, then this CTA's data reads
             s_go = go;
         }
-        __syncthreads();
+        __syncthreads();       // (also publishes the ring's slots)
         if (!s_go) return;
-        if (threadIdx.x == 0 && i + gridDim.x < nitems) {
-            const unsigned w = items[i + gridDim.x].wait;
-            pre = w != kQNone ? q_load(counters + w) : 0;
+        const int next = slot == 2 ? 0 : slot + 1;
+        if (threadIdx.x == 0) {
+            fetch(i + 2 * G, next == 2 ? 0 : next + 1);   // the slot of the item before this one
+            if (i + G < nitems) {
+                const unsigned w = s_item[next].wait;
+                pre = w != kQNone ? q_load(counters + w) : 0;
+                aborted = q_load(abort_flag);
+            }
         }
+        const QItem it = s_item[slot];
         const QGroup &g = prm.g[it.group];
         if (it.op == (Backward ? QOP_C2R : QOP_R2C)) q_run_half<Backward>(Half{}, it.fam, g, it.a, it.b, sm);
         else q_run_strided<Backward>(Full{}, it.op, it.fam, g, it.a, it.b, sm);
+        if (threadIdx.x == 0) cp_async_wait<0>();
         __syncthreads();   // every thread's stores are issued, every shared read is done
         if (threadIdx.x == 0 && it.signal != kQNone) {
             __threadfence();   // release side: the CTA's stores before the increment
             atomicAdd(counters + it.signal, 1u);
         }
+        slot = next;
     }
 }
 
