@@ -251,14 +251,14 @@ template <typename V, typename CT = V> struct GlobalLines {
         return l < valid ? Conv<CT, V>::in(base[l * n + p], bad) : czero<CT>();
     }
 };
-template <typename V, typename CT = V> struct GlobalLinesOut {
+template <typename V, typename CT = V, bool Scaled = true> struct GlobalLinesOut {
     V *base;
     int n;
     int valid;
-    typename RealOf<CT>::T scale;  // 1 forward, 1/N for the last backward store
+    typename RealOf<CT>::T scale;  // 1/N for the last backward store (not Scaled: ignored)
     __device__ __forceinline__ void operator()(int l, int p, CT v) const
     {
-        if (l < valid) base[l * n + p] = Conv<CT, V>::out(cscale(v, scale));
+        if (l < valid) base[l * n + p] = Conv<CT, V>::out(Scaled ? cscale(v, scale) : v);
     }
 };
 

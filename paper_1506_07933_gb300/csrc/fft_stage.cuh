@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
     const V *in0 = in + (d.blk && d.blk_in ? lb : b0) * n;
     V *out0 = out + (d.blk && d.blk_out ? lb : b0) * n;
     const GlobalLines<V> src{in0, n, valid};
-    const GlobalLinesOut<V> dst{out0, n, valid, scale};
+    const GlobalLinesOut<V, V, (S > 0)> dst{out0, n, valid, scale};   // the forward transform is unscaled
     const MapButterflyFast map{};
     if constexpr (F::generic) {
         run_generic<S, false, false, F::split>(d, tw, sm, lines, 0, map, src, dst);
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
             if (d.twdf) {
                 DfFlags bad;
                 const GlobalLines<V, dcx> sdf{in0, n, valid, &bad};
-                const GlobalLinesOut<V, dcx> ddf{out0, n, valid, dfl(scale)};
+                const GlobalLinesOut<V, dcx, (S > 0)> ddf{out0, n, valid, dfl(scale)};
                 const ContigTile<dcx, F> tdf{reinterpret_cast<dcx *>(sm)};
                 if (df_stage<typename F::plan, S, false>((const dcx *)d.twdf, lines, map, sdf, tdf, ddf, bad)) return;
             }
@@ -502,16 +502,15 @@ __device__ __forceinline__ unsigned dynamic_smem_bytes()
 template <typename V, typename CT, class Tile>
 __device__ __forceinline__ void r2c_post(const Tile &tile, V *o, const CT *post_tw, int M, int ld, int valid)
 {
-    using T = typename RealOf<CT>::T;
     const int half = M / 2 + 1;
     for (int idx = threadIdx.x; idx < valid * half; idx += blockDim.x) {
         const int l = idx / half;
         const int k = idx - l * half;
         const CT zk = tile(l, k);
         const CT zm = cconj(tile(l, k == 0 ? 0 : M - k));
-        const CT e = cscale(cadd(zk, zm), T(0.5));
+        const CT s = cadd(zk, zm), e = cmk<CT>(half_of(s.x), half_of(s.y));
         const CT dd = csub(zk, zm);
-        const CT od = cmk<CT>(T(0.5) * dd.y, T(-0.5) * dd.x);  // (zk - zm) / (2i)
+        const CT od = cmk<CT>(half_of(dd.y), -half_of(dd.x));  // (zk - zm) / (2i)
         const CT t = cmul(od, ldgc(post_tw + k));
         V *line = o + l * ld;
         line[k] = Conv<CT, V>::out(cnorm(cadd(e, t)));
@@ -531,7 +530,6 @@ __device__ __forceinline__ bool r2c_post_fixed_k(const Tile &tile, V *o, const C
     if constexpr (M % 2 != 0) {
         return false;
     } else {
-        using T = typename RealOf<CT>::T;
         constexpr int H = M / 2;
         const int nthr = blockDim.x;
         if (H > nthr || nthr % H != 0) return false;
@@ -542,9 +540,9 @@ __device__ __forceinline__ bool r2c_post_fixed_k(const Tile &tile, V *o, const C
             V *line = o + l * ld;
             const CT zk = tile(l, k);
             const CT zm = cconj(tile(l, k == 0 ? 0 : M - k));
-            const CT e = cscale(cadd(zk, zm), T(0.5));
+            const CT s = cadd(zk, zm), e = cmk<CT>(half_of(s.x), half_of(s.y));
             const CT dd = csub(zk, zm);
-            const CT od = cmk<CT>(T(0.5) * dd.y, T(-0.5) * dd.x);  // (zk - zm) / (2i)
+            const CT od = cmk<CT>(half_of(dd.y), -half_of(dd.x));  // (zk - zm) / (2i)
             const CT t = cmul(od, w);
             line[k] = Conv<CT, V>::out(cnorm(cadd(e, t)));
             line[k == 0 ? M : M - k] = Conv<CT, V>::out(cnorm(cconj(csub(e, t))));
@@ -766,10 +764,11 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
 #define AFFT_LINE_PLANS_F64_C(X) X(256, 16, 16) X(384, 6, 8, 8)
 #define AFFT_LINE_PLANS_F64_D(X) X(512, 8, 8, 8) X(1024, 8, 8, 4, 4)
 #define AFFT_LINE_PLANS_F64_E(X) X(2048, 16, 16, 8) X(4096, 16, 16, 16)
-// complex128 lengths whose strided stages are faster with another sequence than their contiguous
-// ones (128 points: N1/N0 of 4 x 128^3 r2c 78/66 -> 66/62 us, but its r2c / c2r lines 172/183 ->
-// 172/192 us; 256 points: N1/N0 of 256^3 c2c 252/245 -> 234/235 us, its c2r lines 1345 -> 1413 us)
-#define AFFT_STRIDED_PLANS_F64(X) X(128, 8, 4, 4) X(256, 8, 8, 4)
+// complex128 lengths whose strided and r2c / c2r stages are faster with another sequence than their
+// contiguous c2c lines (128 points: N1/N0 of 4 x 128^3 r2c 78/66 -> 66/62 us; 256 points: N1/N0 of
+// 256^3 c2c 252/245 -> 234/235 us, but its c2c lines 296 -> 312 us;
+// r2c / c2r lines of 512^3 1311/1345 -> 1289/1241 us with the c2r kernel on twice the threads)
+#define AFFT_OTHER_PLANS_F64(X) X(128, 8, 4, 4) X(256, 8, 8, 4)
 #define AFFT_SPLIT_LINE_PLANS(X)                                                                    \
     X(16, 16) X(32, 16, 2) X(48, 16, 3) X(64, 16, 4) X(80, 16, 5) X(96, 16, 3, 2) X(128, 16, 8)     \
     X(160, 16, 5, 2) X(192, 16, 4, 3) X(256, 16, 16) X(384, 16, 8, 3) X(512, 16, 16, 2)             \
