@@ -155,8 +155,8 @@ bool four_step_split(int64_t n, int &na, int &nb)
     return false;
 }
 
-// The kernels of a line of n points (c2c_lines: contiguous complex lines, unsplit).
-const KernelSet *lookup_kernels(int precision, int64_t n, bool c2c_lines)
+// The kernels of a line of n points (contiguous: on the contiguous axis, unsplit).
+const KernelSet *lookup_kernels(int precision, int64_t n, bool contiguous)
 {
     if (precision == AFFT_F32_SPLIT) {
         // split-precision sequences where the length has radix-16 passes; the FP32 kernels
@@ -167,8 +167,8 @@ const KernelSet *lookup_kernels(int precision, int64_t n, bool c2c_lines)
             if (const KernelSet *k = smooth_kernels_f32((int)n)) return k;
         return generic_kernels_split();
     }
-    if (precision == AFFT_F64 && !c2c_lines)
-        if (const KernelSet *k = other_kernels_f64((int)n)) return k;
+    if (precision == AFFT_F64 && !contiguous)
+        if (const KernelSet *k = strided_kernels_f64((int)n)) return k;
     const KernelSet *k = precision == AFFT_F64 ? spec_kernels_f64((int)n) : spec_kernels_f32((int)n);
     if (!k) k = precision == AFFT_F64 ? smooth_kernels_f64((int)n) : smooth_kernels_f32((int)n);
     if (k) return k;
@@ -1426,7 +1426,7 @@ int afft_plan_create_axes(afft_plan **out, const int64_t n[3], int64_t batch, in
         FourStep &f = p->four[a];
         f.on = split_a[a] > 0;
         const int64_t first = f.on ? split_b[a] : len[a];   // the first (or only) DFT length
-        p->ax[a].ks = lookup_kernels(precision, first, a == 2 && !f.on && kind == AFFT_C2C);
+        p->ax[a].ks = lookup_kernels(precision, first, a == 2 && !f.on);
         p->ax[a].tw_base = (int)tm.size();
         build_desc(first, p->ax[a].ks, p->ax[a].desc, tm, tl);
         if (f.on) {

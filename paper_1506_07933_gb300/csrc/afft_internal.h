@@ -199,9 +199,9 @@ struct KernelSet {
 // Specialised kernels for line length n, or nullptr.
 const KernelSet *spec_kernels_f32(int n);
 const KernelSet *spec_kernels_f64(int n);
-// The kernels of AFFT_OTHER_PLANS_F64 (lengths whose strided and r2c / c2r stages prefer another
-// radix sequence than their contiguous c2c lines; all but the c2c ones), or nullptr.
-const KernelSet *other_kernels_f64(int n);
+// The strided kernels of AFFT_STRIDED_PLANS_F64 (lengths whose strided stages prefer another radix
+// sequence than their contiguous ones; no contiguous kernels), or nullptr.
+const KernelSet *strided_kernels_f64(int n);
 // The families of AFFT_SMOOTH_PLANS (the other 2/3/5-smooth lengths up to 1024), or nullptr.
 const KernelSet *smooth_kernels_f32(int n);
 const KernelSet *smooth_kernels_f64(int n);

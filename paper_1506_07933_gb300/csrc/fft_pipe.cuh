@@ -1056,8 +1056,8 @@ __global__ void __launch_bounds__(PoissonShape<P, V>::threads, PoissonShape<P, V
     }
 }
 
-// The kernels of one family as untyped entry points for the host (Lines: with the contiguous c2c ones).
-template <class F, typename V, bool Lines = true> KernelSet kernel_set(int n, int npass, const int *radix)
+// The kernels of one family as untyped entry points for the host (Contig: with the contiguous ones).
+template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, int npass, const int *radix)
 {
     KernelSet k{};
     k.n = n;
@@ -1065,12 +1065,12 @@ template <class F, typename V, bool Lines = true> KernelSet kernel_set(int n, in
     for (int i = 0; i < npass && i < kMaxPasses; ++i) k.radix[i] = radix[i];
     k.fn[KS_STRIDED_FWD] = (const void *)k_strided<F, -1, V>;
     k.fn[KS_STRIDED_BWD] = (const void *)k_strided<F, +1, V>;
-    if constexpr (Lines) {
+    if constexpr (Contig) {
         k.fn[KS_CONTIG_FWD] = (const void *)k_contig<F, -1, V>;
         k.fn[KS_CONTIG_BWD] = (const void *)k_contig<F, +1, V>;
+        k.fn[KS_R2C] = (const void *)k_r2c<F, V>;
+        k.fn[KS_C2R] = (const void *)k_c2r<F, V>;
     }
-    k.fn[KS_R2C] = (const void *)k_r2c<F, V>;
-    k.fn[KS_C2R] = (const void *)k_c2r<F, V>;
     k.max_threads = F::template threads<V>();
     k.generic = F::generic;
     k.split = F::split;

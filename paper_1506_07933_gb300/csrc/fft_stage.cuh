@@ -764,11 +764,10 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
 #define AFFT_LINE_PLANS_F64_C(X) X(256, 16, 16) X(384, 6, 8, 8)
 #define AFFT_LINE_PLANS_F64_D(X) X(512, 8, 8, 8) X(1024, 8, 8, 4, 4)
 #define AFFT_LINE_PLANS_F64_E(X) X(2048, 16, 16, 8) X(4096, 16, 16, 16)
-// complex128 lengths whose strided and r2c / c2r stages are faster with another sequence than their
-// contiguous c2c lines (128 points: N1/N0 of 4 x 128^3 r2c 78/66 -> 66/62 us; 256 points: N1/N0 of
-// 256^3 c2c 252/245 -> 234/235 us, but its c2c lines 296 -> 312 us;
-// r2c / c2r lines of 512^3 1311/1345 -> 1289/1241 us with the c2r kernel on twice the threads)
-#define AFFT_OTHER_PLANS_F64(X) X(128, 8, 4, 4) X(256, 8, 8, 4)
+// complex128 lengths whose strided stages are faster with another sequence than their contiguous
+// ones (128 points: N1/N0 of 4 x 128^3 r2c 78/66 -> 64/59 us, but its c2c lines lose; 256 points:
+// N1/N0 of 256^3 c2c 252/245 -> 223/225 us, but its c2c lines 296 -> 312 us)
+#define AFFT_STRIDED_PLANS_F64(X) X(128, 8, 4, 4) X(256, 8, 8, 4)
 #define AFFT_SPLIT_LINE_PLANS(X)                                                                    \
     X(16, 16) X(32, 16, 2) X(48, 16, 3) X(64, 16, 4) X(80, 16, 5) X(96, 16, 3, 2) X(128, 16, 8)     \
     X(160, 16, 5, 2) X(192, 16, 4, 3) X(256, 16, 16) X(384, 16, 8, 3) X(512, 16, 16, 2)             \

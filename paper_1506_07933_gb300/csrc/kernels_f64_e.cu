@@ -1,7 +1,7 @@
 // kernels_f64_e.cu -- the double2 specialised families of the line lengths in
 // AFFT_LINE_PLANS_F64_E (the complex128 instantiations are the slowest to compile,
-// so they are split over five translation units), and the sets without c2c lines of
-// AFFT_OTHER_PLANS_F64.
+// so they are split over five translation units), and the strided-only sets of
+// AFFT_STRIDED_PLANS_F64.
 #include "kernel_tables.cuh"
 
 namespace afft {
@@ -19,9 +19,9 @@ const KernelSet *spec_kernels_f64_e(int n)
     afft::kernel_set<afft::Spec<afft::LinePlan<N, ##__VA_ARGS__>>, double2, false>(                   \
         N, afft::LinePlan<N, ##__VA_ARGS__>::npass, afft::RadicesOf<afft::LinePlan<N, ##__VA_ARGS__>>::value),
 
-const KernelSet *other_kernels_f64(int n)
+const KernelSet *strided_kernels_f64(int n)
 {
-    static const KernelSet table[] = {AFFT_OTHER_PLANS_F64(AFFT_X)};
+    static const KernelSet table[] = {AFFT_STRIDED_PLANS_F64(AFFT_X)};
     return find_set(table, n);
 }
 
