@@ -88,7 +88,8 @@ template <int LG, bool Define, typename V> struct DefineBoth<MapLineFastC<LG, De
 // 320 points 77 -> 73 us; on row-pair tiles it lost (400 points 271 -> 297 us).
 constexpr int kPipeSmemCap = 200 * 1024;
 
-template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPairs = false, bool DefinePairs = false> struct PipeShape {
+template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPairs = false,
+          bool DefinePairs = P::define_pairs> struct PipeShape {
     static constexpr bool define_pairs = DefinePairs;   // pair passes define their values (DefineBoth)
     static constexpr int row_lines = 128 / (int)sizeof(V);
     __host__ __device__ static constexpr int lines_for(int l)
@@ -210,7 +211,7 @@ template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPai
 };
 
 // Row-pair tiles (k_strided_pipe_rp) carry at most 16 values per thread at every length.
-template <class P> using RpShape = PipeShape<P, float2, 16, true>;
+template <class P> using RpShape = PipeShape<P, float2, 16, true, false>;
 // Fused Poisson tiles run twice the passes in one loop: their pair passes define their values.
 template <class P, typename V> using PoissonShape = PipeShape<P, V, P::smooth ? 20 : 16, false, true>;
 
@@ -370,8 +371,8 @@ __device__ __forceinline__ void scratch_passes(Seq<R, Rest...>, float2 *C, const
     constexpr bool Global = sizeof...(Rest) == 0;
     constexpr int LG = Sh::lg, NT = Sh::threads, B = Sh::covering(R);
     if constexpr (Sh::pairs(R)) {
-        if constexpr (Global) pair_pass<R, S, N, Ns, LG, NT, B, false, true>(C, tw + TwOff, out.pair);
-        else pair_pass<R, S, N, Ns, LG, NT, B, true, true>(C, tw + TwOff, PairSmemOut<LG>{C});
+        if constexpr (Global) pair_pass<R, S, N, Ns, LG, NT, B, false, true, Sh::define_pairs>(C, tw + TwOff, out.pair);
+        else pair_pass<R, S, N, Ns, LG, NT, B, true, true, Sh::define_pairs>(C, tw + TwOff, PairSmemOut<LG>{C});
     } else {
         const SmemRowsC<float2, LG> rows{C};
         if constexpr (Global)
@@ -1085,7 +1086,8 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
         // single-buffered kernel with the same rows, so it keeps the non-pipelined kernel.
         if constexpr (F::plan::smooth) {
             // TMA tiles alone (rows that no tensor map covers take k_strided), one row-pair form
-            // (early release when every pass works on column pairs) and no blocked layout
+            // and no blocked layout (early release of row-pair tiles measured up to 14% slower at these
+            // lengths, 360 points 266 -> 302 us, and at best 5% faster, 180 points 248 -> 237 us, on 600 MB)
             using P = typename F::plan;
             using Sh = PipeShape<P, V>;
             if constexpr (Sh::tma_ok) {
@@ -1097,10 +1099,9 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
                 k.poisson[0] = (const void *)k_poisson_pipe<P, V, true>;
                 k.poisson_smem = Sh::smem_poisson;
                 if constexpr (Sh::rp_ok) {
-                    constexpr bool early = P::npass >= 2 && RpShape<P>::all_pairs;
                     k.pipe_threads_rp = RpShape<P>::threads;
-                    k.pipe_rp[0] = (const void *)k_strided_pipe_rp<P, -1, early>;
-                    k.pipe_rp[1] = (const void *)k_strided_pipe_rp<P, +1, early>;
+                    k.pipe_rp[0] = (const void *)k_strided_pipe_rp<P, -1>;
+                    k.pipe_rp[1] = (const void *)k_strided_pipe_rp<P, +1>;
                     k.pipe_smem_rp = Sh::smem_rp;
                 }
             }

@@ -17,11 +17,11 @@
 // the spatial xyz layout (the paper's local transpose back to xyz is free).
 //
 // Two implementations:
-//  * specialised kernels, one per line length in AFFT_LINE_PLANS: the radix
+//  * specialised kernels, one per line length in AFFT_LINE_PLANS and AFFT_SMOOTH_PLANS: the radix
 //    sequence is a compile-time list, the first pass reads the tile straight
 //    from global memory and the last pass writes it straight back (both
 //    coalesced), and the passes in between exchange through shared memory;
-//  * a generic kernel for every other length: the tile is staged through
+//  * a generic kernel for every other length (above 1024): the tile is staged through
 //    shared memory and each pass is a separate (non-inlined) function chosen
 //    at run time by its radix.
 #pragma once
@@ -127,8 +127,27 @@ template <int N, int... Rs> struct LinePlan {
     template <int R0, int... R> __host__ __device__ static constexpr bool pad_for(Seq<R0, R...>) { return R0 % 4 == 0; }
     __host__ __device__ static constexpr bool pad_for(Seq<>) { return false; }
     static constexpr bool pad = pad_for(Seq<Rs...>{});   // contiguous tiles: see SmemTile
+    static constexpr bool define_pairs = false;          // see smooth_define_pairs
     using seq = Seq<Rs...>;
 };
+
+// Smooth lengths whose complex64 single-row tiles define the values of their column-pair passes too
+// (see DefineBoth): where several passes leave threads idle the undefined values cost registers,
+// elsewhere the second branch does.  Measured at every length on 600 MB, undefined -> defined: 125
+// 250 -> 214 us, 162 254 -> 212, 200 260 -> 197, 216 239 -> 205, 250 265 -> 203, 270 322 -> 209, 300
+// 329 -> 272, 375 309 -> 276, 400 300 -> 240, 432 299 -> 226, 486 263 -> 249, 540 283 -> 233, 768
+// 265 -> 253, 972 284 -> 275; the other lengths are within 2% or slower (36 193 -> 218, 50 191 -> 213,
+// 450 236 -> 249, 600 264 -> 281).
+__host__ __device__ constexpr bool smooth_define_pairs(int n)
+{
+    switch (n) {
+    case 125: case 162: case 200: case 216: case 250: case 270: case 300: case 375: case 400: case 432:
+    case 486: case 540: case 768: case 972:
+        return true;
+    default:
+        return false;
+    }
+}
 
 // A length of AFFT_SMOOTH_PLANS: complex128 lines compute in FP64 (these lengths always did, and
 // float-float would give up the last four of its 52 bits), and only the kernels a plan can reach
@@ -136,6 +155,7 @@ template <int N, int... Rs> struct LinePlan {
 template <int N, int... Rs> struct SmoothPlan : LinePlan<N, Rs...> {
     static constexpr bool df = false;
     static constexpr bool smooth = true;
+    static constexpr bool define_pairs = smooth_define_pairs(N);
 };
 
 // One pass of a specialised sequence: radix_pass, or with Split (complex64

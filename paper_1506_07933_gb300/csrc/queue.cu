@@ -272,9 +272,9 @@ int afft_queue_create(afft_queue **out, int nplans, afft_plan *const *plans)
     }
     for (int dir = 0; dir < 2 && st == AFFT_OK; ++dir) {
         // a dependency emitted two rounds of the grid earlier has usually finished; fields begun
-        // but not finished are kept to 96 MB (of the 126 MB L2).  Measured on the 200-field
-        // workload, forward: one round and 48 MB 8.1 ms, two rounds and 96 MB 6.6 ms
-        const std::vector<QItem> items = order_items(q->groups, dir == 1, nc, 2 * q->grid[dir], 96.0 * (1 << 20));
+        // but not finished are kept to 160 MB.  Measured on the 200-field workload, round trip: 48 MB
+        // 7.79 ms, 96 MB 7.00, 160 MB 6.75, more the same; one round 6.85, four 7.02 ms
+        const std::vector<QItem> items = order_items(q->groups, dir == 1, nc, 2 * q->grid[dir], 160.0 * (1 << 20));
         q->nitems[dir] = (unsigned)items.size();
         if (cudaMalloc(&q->d_items[dir], items.size() * sizeof(QItem)) != cudaSuccess) {
             q->d_items[dir] = nullptr;
