@@ -67,13 +67,21 @@ __host__ __device__ constexpr int bmax_for_radix(int r)
 
 // Radix passes for a line of n points of the generic family: the fewest passes of radices up to
 // 16 (every pass is a round trip through shared memory), and among those the smallest largest
-// radix, then the smallest sum, in descending order.  Writes at most kMaxPasses radices to r and
-// returns their number (0 for n == 1, -1 when n is not 2/3/5-smooth).
+// radix, then the smallest sum, in descending order.  A generic CTA has kGenericThreads threads and
+// holds at least one line, so radices whose butterflies of one line do not fit it are left out (9
+// carries one butterfly per thread where 3 carries five: 2430 points take 15 6 3 3 3, not 9 9 6 5);
+// the three lengths that no sequence fits (3888, 4000, 4050) get one that the launch shapes refuse.
+// Writes at most kMaxPasses radices to r and returns their number (0 for n == 1, -1 when n is not
+// 2/3/5-smooth).
+constexpr int kGenericThreads = 256;
+
 inline int radix_sequence(long long n, int *r)
 {
     static constexpr int kRadices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
     if (n == 1) return 0;
     struct Search {
+        long long n;
+        bool fit;                  // only radices that fit the CTA
         int best[kMaxPasses], cur[kMaxPasses], best_max = 1 << 30, best_sum = 1 << 30;
         void go(long long m, int left, int at, int hi, int sum)
         {
@@ -86,19 +94,23 @@ inline int radix_sequence(long long n, int *r)
             }
             for (int R : kRadices) {
                 if (R > hi || m % R != 0) continue;
+                if (fit && n > (long long)kGenericThreads * R * bmax_for_radix(R)) continue;
                 cur[at] = R;
                 go(m / R, left - 1, at + 1, R, sum + R);
             }
         }
     };
-    for (int k = 1; k <= 6; ++k) {   // lines of at most 4096 points need at most five (3125 = 5^5)
-        Search s;
-        s.go(n, k, 0, 16, 0);
-        if (s.best_sum < (1 << 30)) {
-            for (int i = 0; i < k; ++i) r[i] = s.best[i];
-            return k;
+    for (const bool fit : {true, false})
+        for (int k = 1; k <= 8; ++k) {   // lines of at most 4096 points need at most seven
+            Search s;
+            s.n = n;
+            s.fit = fit;
+            s.go(n, k, 0, 16, 0);
+            if (s.best_sum < (1 << 30)) {
+                for (int i = 0; i < k; ++i) r[i] = s.best[i];
+                return k;
+            }
         }
-    }
     return -1;
 }
 

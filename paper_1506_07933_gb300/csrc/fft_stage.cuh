@@ -363,7 +363,7 @@ struct Generic {
     static constexpr bool generic = true;
     static constexpr bool split = false;
     using plan = LinePlan<0>;
-    template <typename V> static constexpr int threads() { return 256; }
+    template <typename V> static constexpr int threads() { return kGenericThreads; }
     static constexpr int min_blocks = 2;
 };
 // Generic complex64 kernels of split-precision plans: radix-16 passes on the
@@ -372,7 +372,7 @@ struct GenericSplit {
     static constexpr bool generic = true;
     static constexpr bool split = true;
     using plan = LinePlan<0>;
-    template <typename V> static constexpr int threads() { return 256; }
+    template <typename V> static constexpr int threads() { return kGenericThreads; }
     static constexpr int min_blocks = 1;
 };
 

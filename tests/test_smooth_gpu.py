@@ -20,7 +20,8 @@ def smooth(n):
 MAIN = {2, 4, 8, 16, 24, 32, 48, 60, 64, 80, 96, 120, 128, 160, 192, 256, 384, 512, 1024}
 LENGTHS = [n for n in range(2, 1025) if smooth(n) and n not in MAIN]
 # five-smooth lengths of the generic kernels with radices 6, 9, 10, 12 and 15 among their passes
-GENERIC = [1080, 1125, 1458, 1728, 3125]
+# (2430 ... 3750: lengths whose shortest sequences do not fit a CTA)
+GENERIC = [1080, 1125, 1458, 1728, 3125, 2430, 2592, 2916, 3000, 3200, 3240, 3456, 3645, 3750]
 # FP64 lines of these lengths compute in FP64: a length-n FFT of log2(n) <= 12 levels stays within a
 # few eps sqrt(log2 n), far below the float-float kernels' 1e-14
 TOL = {"f32": 2e-6, "f64": 4e-15}
