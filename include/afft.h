@@ -90,7 +90,7 @@ enum {
 /*
  * Create a plan for an n[0] x n[1] x n[2] transform (AccFFT Section 1: the
  * library takes an N0 x N1 x N2 array).  Factors each axis into radix
- * 16/8/4/2/3/5 passes (the Cooley-Tukey reduction of Section 2), computes
+ * 2 ... 16 passes (of 2, 3, 5 and their products; the Cooley-Tukey reduction of Section 2), computes
  * the twiddle tables in FP64 on the current device, and allocates the
  * workspace.  Each n[i] must be >= 1 with prime factors in {2, 3, 5}.  A line
  * longer than 4096 points (the longest one CTA transforms) is split four-step,
