@@ -36,6 +36,9 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 // kernel of the stream launch as soon as every CTA of this one has started, then waits until the
 // previous kernel has finished and its writes are visible.  Only tables that no stage writes (the
 // twiddles) may be read before it.  Returns at once in a kernel launched without the attribute.
+// The stage's data changes while the kernel already runs, so a kernel that calls this must not
+// declare it `const __restrict__`: that allows loads through the non-coherent path, which are
+// defined only for data constant over the kernel's lifetime and which no asm clobber orders.
 __device__ __forceinline__ void stage_begin()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

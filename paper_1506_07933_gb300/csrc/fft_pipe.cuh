@@ -426,7 +426,7 @@ __device__ __forceinline__ bool pipe_df(Seq<R0, Rest...>, double2 *X, double2 *C
 template <class P, int S, typename V, bool TMA, bool Split = false, bool Blocked = false>
 __global__ void __launch_bounds__(PipeShape<P, V>::threads, Split ? PipeShape<P, V>::min_blocks_split
                                                                   : PipeShape<P, V>::min_blocks)
-    k_strided_pipe(const V *__restrict__ in, V *out, const __grid_constant__ CUtensorMap tmap,
+    k_strided_pipe(const V *in, V *out, const __grid_constant__ CUtensorMap tmap,
                    const V *__restrict__ tw, long long W, long long tiles_per_outer, long long ntiles,
                    unsigned *err, const void *twdf, const unsigned *mma, int rev)
 {
@@ -692,7 +692,7 @@ __device__ __forceinline__ void rp_early_passes(Seq<R0, Rest...>, const float2 *
 // (two tile loads in flight during the other passes), as k_strided_pipe does.
 template <class P, int S, bool Early = false>
 __global__ void __launch_bounds__(RpShape<P>::threads, RpShape<P>::min_blocks_rp)
-    k_strided_pipe_rp(const float2 *__restrict__, float2 *out, const __grid_constant__ CUtensorMap tmap,
+    k_strided_pipe_rp(const float2 *, float2 *out, const __grid_constant__ CUtensorMap tmap,
                       const float2 *__restrict__ tw, long long W, long long tiles_per_outer, long long ntiles,
                       unsigned *err, const void *, const unsigned *, int rev)
 {
@@ -932,7 +932,7 @@ __device__ __forceinline__ bool poisson_df(Seq<R0, Rest...>, double2 *X, double2
 
 template <class P, typename V, bool TMA>
 __global__ void __launch_bounds__(PoissonShape<P, V>::threads, PoissonShape<P, V>::min_blocks_poisson)
-    k_poisson_pipe(const V *__restrict__ in, V *out, const __grid_constant__ CUtensorMap tmap,
+    k_poisson_pipe(const V *in, V *out, const __grid_constant__ CUtensorMap tmap,
                    const V *__restrict__ tw, long long W, long long tiles_per_outer, long long ntiles,
                    unsigned *err, const void *twdf, int n1, int nhp, int nh, int rev,
                    const V *__restrict__ twr, const void *twrdf)

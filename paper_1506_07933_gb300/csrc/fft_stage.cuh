@@ -385,7 +385,7 @@ template <typename V, class F> using ContigTile = SmemTile<V, F::plan::n, F::pla
 // takes `lines` adjacent columns of one outer slab.
 template <class F, int S, typename V>
 __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
-    k_strided(const V *__restrict__ in, V *out, const __grid_constant__ StageDesc d,
+    k_strided(const V *in, V *out, const __grid_constant__ StageDesc d,
               const V *__restrict__ tw, long long W, long long tiles_per_outer, int log2_lines)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
 // Contiguous axis, complex to complex (x scale at the store).
 template <class F, int S, typename V>
 __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
-    k_contig(const V *__restrict__ in, V *out, const __grid_constant__ StageDesc d,
+    k_contig(const V *in, V *out, const __grid_constant__ StageDesc d,
              const V *__restrict__ tw, long long nlines, int lines, typename RealOf<V>::T scale)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -579,7 +579,7 @@ __device__ __forceinline__ bool r2c_post_fixed_k(const Tile &tile, V *o, const C
 //   O = (Z[k] - conj Z[M-k]) / (2i),  Z[M] = Z[0].
 template <class F, typename V>
 __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
-    k_r2c(const typename RealOf<V>::T *__restrict__ in, V *out, const __grid_constant__ StageDesc d,
+    k_r2c(const typename RealOf<V>::T *in, V *out, const __grid_constant__ StageDesc d,
           const V *__restrict__ tw, const V *__restrict__ post_tw, long long nlines, int lines)
 {
     using T = typename RealOf<V>::T;
@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
 // is stored as the real pair (x[2m], x[2m+1]) times `scale`.
 template <class F, typename V>
 __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
-    k_c2r(const V *__restrict__ in, typename RealOf<V>::T *out, const __grid_constant__ StageDesc d,
+    k_c2r(const V *in, typename RealOf<V>::T *out, const __grid_constant__ StageDesc d,
           const V *__restrict__ tw, const V *__restrict__ post_tw, long long nlines, int lines,
           typename RealOf<V>::T scale)
 {
@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
 // family only: the split serves lines longer than one CTA holds.
 template <int S, typename V, bool Split>
 __global__ void __launch_bounds__(256, 1)
-    k_fourstep(const V *__restrict__ in, V *out, const __grid_constant__ StageDesc d, const V *__restrict__ tw,
+    k_fourstep(const V *in, V *out, const __grid_constant__ StageDesc d, const V *__restrict__ tw,
                const V *__restrict__ wn, long long W, long long tiles_per_outer, int log2_lines, int nb,
                typename RealOf<V>::T scale)
 {
