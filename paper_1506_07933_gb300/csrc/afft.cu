@@ -119,25 +119,6 @@ bool factor_ok(int64_t n)
     return n == 1;
 }
 
-// Radix passes of a split-precision line of the generic family: the power-of-two part as evenly
-// sized radix-16/8/4/2 passes (radix 16 runs on the tensor cores), then one pass per factor 3 and 5.
-std::vector<int> split_radix_plan(int64_t n)
-{
-    std::vector<int> r;
-    int a = 0;
-    while (n % 2 == 0) { n /= 2; ++a; }
-    if (a > 0) {
-        const int passes = (a + 3) / 4;
-        for (int i = 0; i < passes; ++i) {
-            const int bits = a / passes + (i < a % passes ? 1 : 0);
-            r.push_back(1 << bits);
-        }
-    }
-    while (n % 3 == 0) { n /= 3; r.push_back(3); }
-    while (n % 5 == 0) { n /= 5; r.push_back(5); }
-    return r;
-}
-
 // n = n_a n_b with both factors at most kMaxLine, n_a the largest such factor
 // not above sqrt(n); false if no split exists.
 bool four_step_split(int64_t n, int &na, int &nb)
@@ -172,12 +153,18 @@ const KernelSet *lookup_kernels(int precision, int64_t n, bool contiguous)
     const KernelSet *k = precision == AFFT_F64 ? spec_kernels_f64((int)n) : spec_kernels_f32((int)n);
     if (!k) k = precision == AFFT_F64 ? smooth_kernels_f64((int)n) : smooth_kernels_f32((int)n);
     if (k) return k;
+    if (mixed_pays(n, precision == AFFT_F64 ? 16 : 8, contiguous))
+        return precision == AFFT_F64 ? mixed_kernels_f64() : mixed_kernels_f32();
     return precision == AFFT_F64 ? generic_kernels_f64() : generic_kernels_f32();
 }
 
 // Fills desc for length n and the radix sequence `rad`, and appends its twiddle entries (m, L),
-// meaning exp(-2 pi i m / L), to the table lists.
-void build_desc(const std::vector<int> &rad, int64_t n, StageDesc &d, std::vector<int> &tm, std::vector<int> &tl)
+// meaning exp(-2 pi i m / L), to the table lists.  r-major: the threads of a contiguous line take
+// consecutive k, one run of the table per r, at constant distances in compile-time passes; k-major in
+// the generic families, whose run-time r-major distances cost a pass its addresses (2000 points N2 726
+// -> 810 us, 1280 points N0 817 -> 964 us).
+void build_desc(const std::vector<int> &rad, int64_t n, bool k_major, StageDesc &d, std::vector<int> &tm,
+                std::vector<int> &tl)
 {
     std::memset(&d, 0, sizeof d);
     d.n = (int)n;
@@ -190,12 +177,11 @@ void build_desc(const std::vector<int> &rad, int64_t n, StageDesc &d, std::vecto
         d.ns[p] = ns;
         d.tw_off[p] = (int)tm.size() - base;
         if (ns > 1) {
-            // r-major: the threads of a contiguous line take consecutive k, one run of the table per r
-            for (int r = 1; r < R; ++r)
-                for (int k = 0; k < ns; ++k) {
-                    tm.push_back((int)(((long long)r * k) % ((long long)R * ns)));
-                    tl.push_back(R * ns);
-                }
+            for (int i = 0; i < (R - 1) * ns; ++i) {
+                const int r = (k_major ? i % (R - 1) : i / ns) + 1, k = k_major ? i / (R - 1) : i % ns;
+                tm.push_back((int)(((long long)r * k) % ((long long)R * ns)));
+                tl.push_back(R * ns);
+            }
         }
         ns *= R;
     }
@@ -204,26 +190,14 @@ void build_desc(const std::vector<int> &rad, int64_t n, StageDesc &d, std::vecto
 // The same with the radix sequence of the kernels (theirs when specialised).
 void build_desc(int64_t n, const KernelSet *ks, StageDesc &d, std::vector<int> &tm, std::vector<int> &tl)
 {
-    std::vector<int> rad;
-    if (!ks->generic) rad.assign(ks->radix, ks->radix + ks->npass);
-    else if (ks == generic_kernels_split()) rad = split_radix_plan(n);
-    else {
-        int r[kMaxPasses];
-        rad.assign(r, r + std::max(0, radix_sequence(n, r)));
-    }
-    build_desc(rad, n, d, tm, tl);
+    int r[kMaxPasses];
+    int np = ks->npass;
+    if (!ks->generic) std::copy(ks->radix, ks->radix + np, r);
+    else np = ks == mixed_kernels_f32() || ks == mixed_kernels_f64() ? radix_sequence(n, r) : basic_sequence(n, r);
+    build_desc(std::vector<int>(r, r + np), n, ks->generic, d, tm, tl);
 }
 
-int required_threads(const StageDesc &d, int lines)
-{
-    long long req = lines;  // copy path (n == 1)
-    for (int p = 0; p < d.npass; ++p) {
-        const long long bf = (long long)lines * (d.n / d.radix[p]);
-        const int per = bmax_for_radix(d.radix[p]);
-        req = std::max(req, (bf + per - 1) / per);
-    }
-    return (int)std::max(32LL, (req + 31) / 32 * 32);
-}
+int required_threads(const StageDesc &d, int lines) { return line_threads(d.radix, d.npass, d.n, lines); }
 
 int ilog2(int v)
 {
@@ -1434,7 +1408,8 @@ int afft_plan_create_axes(afft_plan **out, const int64_t n[3], int64_t batch, in
             f.na = split_a[a];
             f.nb = split_b[a];
             f.a.ks = precision == AFFT_F64 ? generic_kernels_f64()
-                     : precision == AFFT_F32_SPLIT ? generic_kernels_split() : generic_kernels_f32();
+                     : precision == AFFT_F32_SPLIT ? generic_kernels_split()
+                     : mixed_pays(f.na, 8, false, 255) ? mixed_kernels_f32() : generic_kernels_f32();
             f.a.tw_base = (int)tm.size();
             build_desc(f.na, f.a.ks, f.a.desc, tm, tl);
             f.wn_base = (int)tm.size();
@@ -1452,7 +1427,7 @@ int afft_plan_create_axes(afft_plan **out, const int64_t n[3], int64_t batch, in
         if (!std::equal(back.begin(), back.end(), d.radix)) {
             p->ax[0].twr_base = (int)tm.size();
             StageDesc unused;
-            build_desc(back, d.n, unused, tm, tl);
+            build_desc(back, d.n, false, unused, tm, tl);
         }
     }
     p->post_off = (int)tm.size();

@@ -26,7 +26,9 @@ struct StageDesc {
     int npass;                     // number of radix passes (0 when n == 1)
     int radix[kMaxPasses];         // radix of each pass
     int ns[kMaxPasses];            // product of the radices of the earlier passes
-    int tw_off[kMaxPasses];        // first twiddle of each pass (complex entries)
+    // first twiddle of each pass (complex entries); entry (k, r), k < ns and 1 <= r < radix, of the
+    // pass is at (r - 1) ns + k, or in the k-major tables of the generic families at k (radix - 1) + r - 1
+    int tw_off[kMaxPasses];
     int ld;                        // r2c/c2r stage: stride between half-spectrum lines, in complex
                                    // elements; 0 means compact (M + 1 for a line of M points)
     // FP64 plans: the same twiddle tables as float-float values (hi, lo floats),
@@ -65,7 +67,21 @@ __host__ __device__ constexpr int bmax_for_radix(int r)
     return r >= 16 ? 1 : (r == 3 ? 5 : (r == 5 ? 3 : 16 / r));
 }
 
-// Radix passes for a line of n points of the generic family: the fewest passes of radices up to
+// Radix passes of a generic line of n points: the power-of-two part as evenly sized radix-16/8/4/2
+// passes (radix 16 runs on the tensor cores in split precision), then one pass per factor 3 and 5.
+// Writes at most kMaxPasses radices to r and returns their number (0 for n == 1).
+inline int basic_sequence(long long n, int *r)
+{
+    int k = 0, a = 0;
+    while (n % 2 == 0) { n /= 2; ++a; }
+    const int passes = (a + 3) / 4;
+    for (int i = 0; i < passes; ++i) r[k++] = 1 << (a / passes + (i < a % passes ? 1 : 0));
+    while (n % 3 == 0) { n /= 3; r[k++] = 3; }
+    while (n % 5 == 0) { n /= 5; r[k++] = 5; }
+    return k;
+}
+
+// Radix passes for a line of n points of the mixed generic family: the fewest passes of radices up to
 // 16 (every pass is a round trip through shared memory), and among those the smallest largest
 // radix, then the smallest sum, in descending order.  A generic CTA has kGenericThreads threads and
 // holds at least one line, so radices whose butterflies of one line do not fit it are left out (9
@@ -112,6 +128,65 @@ inline int radix_sequence(long long n, int *r)
             }
         }
     return -1;
+}
+
+// Threads that hold every butterfly of each pass of `lines` lines.
+inline int line_threads(const int *radix, int npass, long long n, int lines)
+{
+    long long req = lines;   // copy path (n == 1)
+    for (int p = 0; p < npass; ++p) {
+        const int per = bmax_for_radix(radix[p]);
+        const long long t = ((long long)lines * (n / radix[p]) + per - 1) / per;
+        req = t > req ? t : req;
+    }
+    return (int)(req < 32 ? 32 : (req + 31) / 32 * 32);
+}
+
+// Whether a generic line of n points runs the mixed family (radix_sequence) or the basic one
+// (basic_sequence); elem: bytes per complex value.  Both were measured at every smooth length from
+// 1080 to 4096 on 320 to 640 MB.
+//  * The mixed sequence must have fewer passes (3125, 3200 and 3456 points, the same passes in both,
+//    lose 2 to 9%; 2000 = 10 8 5 5 against 16 5 5 5 lost 4 to 20%).
+//  * complex64 passes are bound by shared memory and barriers, so their time goes as passes over
+//    points resident per SM, and wide radices give a line fewer threads.  With that quotient up to 1.2
+//    times the basic one the mixed family measured 0.55 to 0.98 (2700 points N2 1074 -> 594 us, N0 1109
+//    -> 784 us; 1440 points N0 1054 -> 800 us); above, lost or equal (1.88: 1920 points N0 701 ->
+//    946 us; 1.5: 1800 points N0 846 -> 1000 us, 1280 points N2 557 -> 600 us).  A strided tile that
+//    halves its columns reads half the bytes per row: its quotient counts 1.25 times (1600 points N0,
+//    1.0 x 1.25, 852 -> 930 us).
+//  * complex128 passes are bound by the FP64 pipe: two radix-9 butterflies with their inner twiddles and
+//    idle lanes cost what four radix-3 passes do (1458 = 9 9 6 3: N2 3475 -> 3690 us, 1215 = 15 9 9: r2c
+//    3884 -> 4150 us); the other lengths measured 0.78 to 1.04 (2592 points N0 3977 -> 3200 us, 1920
+//    points N0 2780 -> 2880 us).
+// regs: registers per thread of the kernel (255 in the four-step kernel, where the same quotient told
+// complex64 halves of 72 and 75 points, 0.67 and measured 0.75 to 0.91 on the transform, from 50, 60
+// and 100, 1.33 and measured 1.22 to 1.36; complex128 ones lose 2 to 7% and stay with the basic family).
+inline bool mixed_pays(long long n, int elem, bool contiguous, int regs = 128)
+{
+    int basic[kMaxPasses], mixed[kMaxPasses];
+    const int nb = basic_sequence(n, basic), nm = radix_sequence(n, mixed);
+    if (nm <= 0 || nm >= nb) return false;
+    if (elem == 16) {
+        if (regs > 128) return false;
+        int nines = 0;
+        for (int p = 0; p < nm; ++p) nines += mixed[p] == 9;
+        return nines < 2;
+    }
+    constexpr int kSmem = 227 * 1024;   // an SM's shared memory
+    int lines[2];
+    double cost[2];
+    for (int m = 0; m < 2; ++m) {
+        const int *r = m ? mixed : basic, np = m ? nm : nb;
+        int l = contiguous ? (int)(4096 / n > 1 ? 4096 / n : 1) : 128 / elem;
+        while (l > 1 && (line_threads(r, np, n, l) > kGenericThreads || n * l * elem > kSmem))
+            l = contiguous ? (l + 1) / 2 : l / 2;
+        const int by_regs = 65536 / (regs * line_threads(r, np, n, l)), by_smem = (int)(kSmem / (n * l * elem + 1024));
+        const int ctas = by_regs < by_smem ? by_regs : by_smem;
+        lines[m] = l;
+        cost[m] = (double)np / ((double)l * (ctas > 1 ? ctas : 1));
+    }
+    if (!contiguous && lines[1] < lines[0]) cost[1] *= 1.25;
+    return cost[1] <= 1.2 * cost[0] * (1 + 1e-9);
 }
 
 // Rows per TMA box when a line of n rows is loaded in boxes of at most 256
@@ -217,9 +292,12 @@ const KernelSet *strided_kernels_f64(int n);
 // The families of AFFT_SMOOTH_PLANS (the other 2/3/5-smooth lengths up to 1024), or nullptr.
 const KernelSet *smooth_kernels_f32(int n);
 const KernelSet *smooth_kernels_f64(int n);
-// Generic kernels (any n whose radix plan the host builds).
+// Generic kernels (any n whose radix plan the host builds): radices of basic_sequence, and with the
+// radices of radix_sequence too (mixed; no Poisson kernel).
 const KernelSet *generic_kernels_f32();
 const KernelSet *generic_kernels_f64();
+const KernelSet *mixed_kernels_f32();
+const KernelSet *mixed_kernels_f64();
 // Generic complex64 kernels whose radix-16 passes run on the tensor cores
 // (split-precision plans), and the device table of their DFT-16 fragments
 // (kSplitTableBytes, written by split_fragments on `stream`).

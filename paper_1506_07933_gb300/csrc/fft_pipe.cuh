@@ -1077,11 +1077,12 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
     k.split = F::split;
     k.contig_pad = F::plan::pad;
     if constexpr (F::generic) {
-        k.four[0] = (const void *)k_fourstep<-1, V, F::split>;
-        k.four[1] = (const void *)k_fourstep<+1, V, F::split>;
-        k.poisson_mult = (const void *)k_poisson_mult<V>;
-    }
-    if constexpr (!F::generic) {
+        if constexpr (!F::mixed || sizeof(V) == 8) {
+            k.four[0] = (const void *)k_fourstep<F, -1, V>;
+            k.four[1] = (const void *)k_fourstep<F, +1, V>;
+        }
+        if constexpr (!F::mixed) k.poisson_mult = (const void *)k_poisson_mult<V>;
+    } else {
         // n = 1024 would need 64-byte tile rows to double-buffer; measured slower than the
         // single-buffered kernel with the same rows, so it keeps the non-pipelined kernel.
         if constexpr (F::plan::smooth) {

@@ -71,8 +71,8 @@ __device__ __forceinline__ void split_scale(float m, float &sc, float &inv)
 // every read of the CTA precedes the barrier, every write follows it).  The
 // CTA covers all lines * n / 16 butterflies with at most 4 groups of 8 per
 // warp (the host sizes CTAs so that threads >= butterflies).  frag: the
-// fragment table of this direction (32 words per lane).
-template <int S, class Map, class Src, class Dst>
+// fragment table of this direction (32 words per lane).  KMajor: as in radix_pass.
+template <int S, bool KMajor = false, class Map, class Src, class Dst>
 __device__ __forceinline__ void mma16_pass(int n, int Ns, const float2 *__restrict__ tw, int lines, const Map &map,
                                            const Src &src, const Dst &dst, const unsigned *__restrict__ frag)
 {
@@ -108,11 +108,11 @@ __device__ __forceinline__ void mma16_pass(int n, int Ns, const float2 *__restri
 #pragma unroll
             for (int t = 0; t < 4; ++t) x[t] = src(l, j + (q + 4 * t) * nb);
             if (Ns > 1) {
-                const float2 *w = tw + j % Ns;
+                const float2 *w = tw + (j % Ns) * (KMajor ? 15 : 1);
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
                     const int r = q + 4 * t;
-                    if (r > 0) x[t] = ctw<S>(x[t], ldgc(w + (r - 1) * Ns));
+                    if (r > 0) x[t] = ctw<S>(x[t], ldgc(w + (r - 1) * (KMajor ? 1 : Ns)));
                 }
             }
         }

@@ -21,9 +21,9 @@
 //    sequence is a compile-time list, the first pass reads the tile straight
 //    from global memory and the last pass writes it straight back (both
 //    coalesced), and the passes in between exchange through shared memory;
-//  * a generic kernel for every other length (above 1024): the tile is staged through
-//    shared memory and each pass is a separate (non-inlined) function chosen
-//    at run time by its radix.
+//  * a generic kernel for every other length (above 1024; in split-precision plans also the
+//    multiples of 16 without a split sequence): the tile is staged through shared memory and each
+//    pass is a separate (non-inlined) function chosen at run time by its radix.
 #pragma once
 
 #include <type_traits>
@@ -66,10 +66,10 @@ template <class Map, typename V> struct DefineBoth { static constexpr bool value
 // Thread t handles butterflies idx = t, t + blockDim.x, ... (at most
 // bmax_for_radix(R) of them; the host sizes the CTA so that suffices).  With
 // InPlace the pass reads everything into registers, waits for the whole CTA,
-// then writes.
+// then writes.  KMajor: the pass's table is k-major (StageDesc).
 
-template <int R, int S, bool InPlace, int NT = 0, int BM = 0, bool TwSmem = false, typename V, class Map, class Src,
-          class Dst>
+template <int R, int S, bool InPlace, int NT = 0, int BM = 0, bool TwSmem = false, bool KMajor = false, typename V,
+          class Map, class Src, class Dst>
 __device__ __forceinline__ void radix_pass(int n, int Ns, const V *__restrict__ tw, int lines,
                                            const Map &map, const Src &src, const Dst &dst)
 {
@@ -92,9 +92,10 @@ __device__ __forceinline__ void radix_pass(int n, int Ns, const V *__restrict__ 
 #pragma unroll
             for (int r = 0; r < R; ++r) v[b][r] = tile_ld(src, l, j, r * nb);
             if (Ns > 1) {
-                const V *t = tw + j % Ns;
+                const V *t = tw + (j % Ns) * (KMajor ? R - 1 : 1);
 #pragma unroll
-                for (int r = 1; r < R; ++r) v[b][r] = ctw<S>(v[b][r], tw_ld<TwSmem>(t + (r - 1) * Ns));
+                for (int r = 1; r < R; ++r)
+                    v[b][r] = ctw<S>(v[b][r], tw_ld<TwSmem>(t + (r - 1) * (KMajor ? 1 : Ns)));
             }
             Dft<R, S, V>::run(v[b]);
         } else if constexpr (DefineBoth<Map, V>::value) {
@@ -266,10 +267,10 @@ __device__ __noinline__ void smem_pass(V *sm, int n, int Ns, const V *tw, int li
 {
     if constexpr (Rows) {
         const SmemRows<V> t{sm, log2_lines};
-        radix_pass<R, S, true>(n, Ns, tw, lines, MapLineFast{log2_lines}, t, t);
+        radix_pass<R, S, true, 0, 0, false, true>(n, Ns, tw, lines, MapLineFast{log2_lines}, t, t);
     } else {
         const SmemLines<V> t{sm, n};
-        radix_pass<R, S, true>(n, Ns, tw, lines, MapButterflyFast{}, t, t);
+        radix_pass<R, S, true, 0, 0, false, true>(n, Ns, tw, lines, MapButterflyFast{}, t, t);
     }
 }
 
@@ -280,41 +281,47 @@ __device__ __noinline__ void smem_mma16(float2 *sm, int n, int Ns, const float2 
 {
     if constexpr (Rows) {
         const SmemRows<float2> t{sm, log2_lines};
-        mma16_pass<S>(n, Ns, tw, lines, MapLineFast{log2_lines}, t, t, frag);
+        mma16_pass<S, true>(n, Ns, tw, lines, MapLineFast{log2_lines}, t, t, frag);
     } else {
         const SmemLines<float2> t{sm, n};
-        mma16_pass<S>(n, Ns, tw, lines, MapButterflyFast{}, t, t, frag);
+        mma16_pass<S, true>(n, Ns, tw, lines, MapButterflyFast{}, t, t, frag);
     }
 }
 
-template <int S, bool Rows, bool Split, typename V>
+template <class F, int S, bool Rows, typename V>
 __device__ __forceinline__ void smem_pass_any(int R, V *sm, int n, int Ns, const V *tw, int lines,
                                               int log2_lines, const unsigned *mma)
 {
     switch (R) {
     case 16:
-        if constexpr (Split && std::is_same<V, float2>::value)
+        if constexpr (F::split && std::is_same<V, float2>::value)
             smem_mma16<S, Rows>(sm, n, Ns, tw, lines, log2_lines, mma + (S < 0 ? 0 : 32 * 32));
         else
             smem_pass<16, S, Rows>(sm, n, Ns, tw, lines, log2_lines);
         break;
-    case 15: smem_pass<15, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
-    case 12: smem_pass<12, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
-    case 10: smem_pass<10, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
-    case 9: smem_pass<9, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 8: smem_pass<8, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
-    case 6: smem_pass<6, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 4: smem_pass<4, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 2: smem_pass<2, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 3: smem_pass<3, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
     case 5: smem_pass<5, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
-    default: break;  // the plan emits only the radices above
+    default:
+        if constexpr (F::mixed) {
+            switch (R) {
+            case 15: smem_pass<15, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+            case 12: smem_pass<12, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+            case 10: smem_pass<10, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+            case 9: smem_pass<9, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+            case 6: smem_pass<6, S, Rows>(sm, n, Ns, tw, lines, log2_lines); break;
+            default: break;
+            }
+        }
+        break;  // the plan emits only the radices above
     }
 }
 
 // Generic stage body: load src -> smem, all passes in smem, store smem -> dst
-// (skipped with LastToSmem).  Split: radix-16 passes on the tensor cores.
-template <int S, bool Rows, bool LastToSmem, bool Split = false, typename V, class Map, class Src, class Dst>
+// (skipped with LastToSmem).  F: the family (split: radix-16 passes on the tensor cores).
+template <class F, int S, bool Rows, bool LastToSmem, typename V, class Map, class Src, class Dst>
 __device__ __forceinline__ void run_generic(const StageDesc &d, const V *tw, V *sm, int lines,
                                             int log2_lines, const Map &map, const Src &src,
                                             const Dst &dst)
@@ -331,7 +338,7 @@ __device__ __forceinline__ void run_generic(const StageDesc &d, const V *tw, V *
     }
     for (int p = 0; p < d.npass; ++p) {
         __syncthreads();
-        smem_pass_any<S, Rows, Split>(d.radix[p], sm, n, d.ns[p], tw + d.tw_off[p], lines, log2_lines, d.mma);
+        smem_pass_any<F, S, Rows>(d.radix[p], sm, n, d.ns[p], tw + d.tw_off[p], lines, log2_lines, d.mma);
     }
     if constexpr (LastToSmem) return;
     __syncthreads();
@@ -362,15 +369,24 @@ template <class Plan, bool Split = false> struct Spec {
 struct Generic {
     static constexpr bool generic = true;
     static constexpr bool split = false;
+    static constexpr bool mixed = false;
     using plan = LinePlan<0>;
     template <typename V> static constexpr int threads() { return kGenericThreads; }
     static constexpr int min_blocks = 2;
+};
+// Generic kernels whose passes may also have radix 6, 9, 10, 12 and 15 (mixed_pays in afft.cu says for
+// which lengths).  A family of its own because the larger switch over passes costs the others: lengths
+// that run the same passes in both measured 2 to 9% slower in this one (complex64 N0 stage of 3125
+// points 905 -> 976 us, of 1920 points 701 -> 743 us on 320 MB).
+struct GenericMixed : Generic {
+    static constexpr bool mixed = true;
 };
 // Generic complex64 kernels of split-precision plans: radix-16 passes on the
 // tensor cores, otherwise as Generic.
 struct GenericSplit {
     static constexpr bool generic = true;
     static constexpr bool split = true;
+    static constexpr bool mixed = false;
     using plan = LinePlan<0>;
     template <typename V> static constexpr int threads() { return kGenericThreads; }
     static constexpr int min_blocks = 1;
@@ -402,7 +418,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
     const GlobalColsOut<V> dst{out + off, W, valid};
     const MapLineFast map{log2_lines};
     if constexpr (F::generic) {
-        run_generic<S, true, false, F::split>(d, tw, sm, lines, log2_lines, map, src, dst);
+        run_generic<F, S, true, false>(d, tw, sm, lines, log2_lines, map, src, dst);
     } else {
         if constexpr (UseDf<F, V>::value) {
             if (d.twdf) {
@@ -439,7 +455,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
     const GlobalLinesOut<V, V, (S > 0)> dst{out0, n, valid, scale};   // the forward transform is unscaled
     const MapButterflyFast map{};
     if constexpr (F::generic) {
-        run_generic<S, false, false, F::split>(d, tw, sm, lines, 0, map, src, dst);
+        run_generic<F, S, false, false>(d, tw, sm, lines, 0, map, src, dst);
     } else {
         if constexpr (UseDf<F, V>::value) {
             if (d.twdf) {
@@ -610,7 +626,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
     // k_c2r does measured 12% slower here, the 16 loads of a thread being in flight together)
     if constexpr (F::generic) {
         const SmemLines<V> tile{sm, M};
-        run_generic<-1, false, true, F::split>(d, tw, sm, lines, 0, map, src, tile);
+        run_generic<F, -1, false, true>(d, tw, sm, lines, 0, map, src, tile);
         __syncthreads();
         r2c_post<V, V>(tile, o, post_tw, M, ld, valid);
     } else {
@@ -645,7 +661,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
     const GlobalLinesOut<V> dst{reinterpret_cast<V *>(out) + b0 * M, M, valid, scale};
     const MapButterflyFast map{};
     if constexpr (F::generic) {
-        run_generic<+1, false, false, F::split>(d, tw, sm, lines, 0, map, src, dst);
+        run_generic<F, +1, false, false>(d, tw, sm, lines, 0, map, src, dst);
     } else {
         // complex64 (not split): the CTA's lines are one contiguous run of valid * (M + 1)
         // elements; when it starts 16-byte aligned it is copied by one bulk copy (TMA) into the
@@ -716,7 +732,7 @@ __global__ void __launch_bounds__(F::template threads<V>(), F::min_blocks)
 // [outer * n_b][n_a][W] (row k_b of each outer line group holds the length-n_b
 // DFT outputs, laid out as n_a rows), the output [outer][n_a n_b][W].  Generic
 // family only: the split serves lines longer than one CTA holds.
-template <int S, typename V, bool Split>
+template <class F, int S, typename V>
 __global__ void __launch_bounds__(256, 1)
     k_fourstep(const V *in, V *out, const __grid_constant__ StageDesc d, const V *__restrict__ tw,
                const V *__restrict__ wn, long long W, long long tiles_per_outer, int log2_lines, int nb,
@@ -734,7 +750,7 @@ __global__ void __launch_bounds__(256, 1)
     const int valid = (int)min((long long)lines, W - c0);
     const FourStepSrc<S, V> src{in + op * (long long)na * W + c0, W, valid, wn, kb};
     const FourStepDst<V> dst{out + (o * (long long)na * nb + kb) * W + c0, (long long)nb * W, valid, scale};
-    run_generic<S, true, false, Split>(d, tw, sm, lines, log2_lines, MapLineFast{log2_lines}, src, dst);
+    run_generic<F, S, true, false>(d, tw, sm, lines, log2_lines, MapLineFast{log2_lines}, src, dst);
 }
 
 // Spectral Poisson multiply on a half spectrum [planes][n1][nhp] (rows of nhp >= nh elements; planes =

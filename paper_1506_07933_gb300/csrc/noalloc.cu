@@ -76,18 +76,6 @@ struct Axis {
     long long blocks, tpo;
 };
 
-int threads_for(const StageDesc &d, int lines)
-{
-    long long req = lines;
-    for (int p = 0; p < d.npass; ++p) {
-        const long long bf = (long long)lines * (d.n / d.radix[p]);
-        const int per = bmax_for_radix(d.radix[p]);
-        if ((bf + per - 1) / per > req) req = (bf + per - 1) / per;
-    }
-    req = (req + 31) / 32 * 32;
-    return (int)(req < 32 ? 32 : req);
-}
-
 // Fills the descriptor (twiddle offsets relative to the axis) and counts its
 // twiddle entries.
 void describe(int64_t n, int precision, Axis &a, int &tw_count)
@@ -103,7 +91,7 @@ void describe(int64_t n, int precision, Axis &a, int &tw_count)
         np = a.ks->npass;
         for (int i = 0; i < np; ++i) rad[i] = a.ks->radix[i];
     } else {
-        np = radix_sequence(n, rad);
+        np = basic_sequence(n, rad);
     }
     a.d.npass = np;
     a.tw_base = tw_count;
@@ -123,7 +111,7 @@ bool shape_strided(Axis &a, long long outer, long long W, size_t elem, size_t ma
     int lines = (int)(128 / elem);
     while (lines > 1 && lines / 2 >= W) lines /= 2;
     for (;;) {
-        const int thr = threads_for(a.d, lines);
+        const int thr = line_threads(a.d.radix, a.d.npass, a.d.n, lines);
         const size_t smem = (size_t)a.d.n * lines * elem;
         if (thr <= a.ks->max_threads && smem <= max_smem) {
             int lg = 0;
@@ -153,7 +141,7 @@ bool shape_contig(Axis &a, long long nlines, size_t elem, size_t max_smem, bool 
     if (even_lines && lines > 1 && (lines & 1)) --lines;
     const int row = (int)(128 / elem);
     for (;;) {
-        const int thr = threads_for(a.d, lines);
+        const int thr = line_threads(a.d.radix, a.d.npass, a.d.n, lines);
         const size_t smem = (size_t)contig_tile_elems(lines * a.d.n, row, a.ks->contig_pad) * elem;
         if (thr <= a.ks->max_threads && smem <= max_smem) {
             a.lines = lines;
@@ -169,11 +157,13 @@ bool shape_contig(Axis &a, long long nlines, size_t elem, size_t max_smem, bool 
     }
 }
 
-// Twiddle tables straight from the descriptors: for each pass with Ns > 1,
-// entry k (R-1) + r-1 = exp(-2 pi i (r k mod R Ns) / (R Ns)); then the c2r
-// table exp(-2 pi i k / n2), k = 0..n2/2.  FP64 sincospi, argument reduced.
+// Twiddle tables straight from the descriptors: for each pass with Ns > 1, entry (k, r) =
+// exp(-2 pi i (r k mod R Ns) / (R Ns)) at (r-1) Ns + k, or in a generic axis' k-major tables at
+// k (R-1) + r-1; then the c2r table exp(-2 pi i k / n2), k = 0..n2/2.  FP64 sincospi, argument
+// reduced.
 struct TwJob {
     int nseg;
+    bool k_major[3 * kMaxPasses];
     int base[3 * kMaxPasses];
     int R[3 * kMaxPasses];
     int Ns[3 * kMaxPasses];
@@ -195,8 +185,9 @@ __global__ void k_noalloc_twiddles(V *tw, const __grid_constant__ TwJob job)
         int s = 0;
         while (s + 1 < job.nseg && i >= job.base[s + 1]) ++s;
         const int local = i - job.base[s];
-        const int r = local / job.Ns[s] + 1;
-        const int k = local - (r - 1) * job.Ns[s];
+        const int R1 = job.R[s] - 1;
+        const int r = (job.k_major[s] ? local % R1 : local / job.Ns[s]) + 1;
+        const int k = job.k_major[s] ? local / R1 : local % job.Ns[s];
         L = job.R[s] * job.Ns[s];
         m = (int)(((long long)r * k) % L);
     }
@@ -265,6 +256,7 @@ int run(const int64_t n[3], int precision, const void *in, void *out, cudaStream
             job.base[job.nseg] = ax[a].tw_base + ax[a].d.tw_off[p];
             job.R[job.nseg] = ax[a].d.radix[p];
             job.Ns[job.nseg] = ax[a].d.ns[p];
+            job.k_major[job.nseg] = ax[a].ks->generic;
             ++job.nseg;
         }
     job.post_base = post_base;
