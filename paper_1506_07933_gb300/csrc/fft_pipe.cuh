@@ -913,20 +913,29 @@ __device__ __forceinline__ void poisson_passes(Seq<R, Rest...>, Seq<Back...>, V 
     }
 }
 
-// FP64 tile in float-float: the first pass converts, as in pipe_df.  Returns false, with X
-// untouched, when some value was out of float-float range.
+// FP64 tile in float-float: the first pass converts, as in pipe_df; where the only pass is the middle
+// one, a copy into C does (in FP64 its few butterflies leave most lanes of the FP64 pipe idle, and so do
+// the divisions: N0 operator of 16 x 1024 x 512 873 -> 224 us, 2 x 2048 x 2048 381 -> 155 us).  Returns
+// false, with X untouched, when some value was out of float-float range.
 template <class Sh, int N, class GOut, int R0, int... Rest>
 __device__ __forceinline__ bool poisson_df(Seq<R0, Rest...>, double2 *X, double2 *C, const dcx *tw, const dcx *twr,
                                            const GOut &gout, const PoissonColumn<N, dcx> &c)
 {
     constexpr int LG = Sh::lg;
+    dcx *const Y = reinterpret_cast<dcx *>(C);
     DfFlags bad;
-    const SmemRowsConvIn<double2, dcx, LG> src{X, &bad};
-    radix_pass<R0, -1, false, Sh::threads, Sh::per_thread(R0)>(N, 1, tw, Sh::lines, typename Sh::map{}, src,
-                                                              SmemRowsC<dcx, LG>{reinterpret_cast<dcx *>(C)});
-    if (!df_tile_ok(bad)) return false;
-    poisson_passes<Sh, N, R0, 0, 1, false>(Seq<Rest...>{}, Seq<R0>{}, reinterpret_cast<dcx *>(X),
-                                           reinterpret_cast<dcx *>(C), tw, twr, gout, c, c);
+    if constexpr (sizeof...(Rest) == 0) {
+        for (int e = threadIdx.x; e < Sh::tile; e += Sh::threads) Y[e] = Conv<dcx, double2>::in(X[e], &bad);
+        if (!df_tile_ok(bad)) return false;
+        poisson_mid<Sh, N, R0, false>(Y, tw, gout, c, c);
+    } else {
+        const SmemRowsConvIn<double2, dcx, LG> src{X, &bad};
+        radix_pass<R0, -1, false, Sh::threads, Sh::per_thread(R0)>(N, 1, tw, Sh::lines, typename Sh::map{}, src,
+                                                                  SmemRowsC<dcx, LG>{Y});
+        if (!df_tile_ok(bad)) return false;
+        poisson_passes<Sh, N, R0, 0, 1, false>(Seq<Rest...>{}, Seq<R0>{}, reinterpret_cast<dcx *>(X), Y, tw, twr, gout,
+                                               c, c);
+    }
     return true;
 }
 
@@ -1021,7 +1030,7 @@ __global__ void __launch_bounds__(PoissonShape<P, V>::threads, PoissonShape<P, V
         };
         const long long c = c0 + (tid & (LINES - 1));
         bool done = false;
-        if constexpr (std::is_same<V, double2>::value && P::df) {
+        if constexpr (std::is_same<V, double2>::value && P::df_poisson) {
             if (twdf) {
                 TileOut<V, dcx> g;
                 g.single = GlobalColFixedOut<V, dcx>{obase, W, c < W ? c : -1};

@@ -124,6 +124,7 @@ template <int N, int... Rs> struct LinePlan {
     static constexpr int n = N;
     static constexpr int npass = sizeof...(Rs);
     static constexpr bool df = npass >= 2;   // complex128 lines compute in float-float (needs two passes)
+    static constexpr bool df_poisson = npass >= 1;   // so does the fused Poisson tile, converted by a copy if need be
     static constexpr bool smooth = false;
     template <int R0, int... R> __host__ __device__ static constexpr bool pad_for(Seq<R0, R...>) { return R0 % 4 == 0; }
     __host__ __device__ static constexpr bool pad_for(Seq<>) { return false; }
@@ -155,6 +156,7 @@ __host__ __device__ constexpr bool smooth_define_pairs(int n)
 // are instantiated (see kernel_set).
 template <int N, int... Rs> struct SmoothPlan : LinePlan<N, Rs...> {
     static constexpr bool df = false;
+    static constexpr bool df_poisson = false;
     static constexpr bool smooth = true;
     static constexpr bool define_pairs = smooth_define_pairs(N);
 };
