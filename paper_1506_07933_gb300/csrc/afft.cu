@@ -452,8 +452,14 @@ int plan_shapes(afft_plan *p)
         ap.pipe_slots = sms * per_sm;   // also what the blocked c2c layout runs with
         // rows far apart: the many CTAs of the plain kernel win in the row-major layout
         const bool far = ks->n >= 1024 && row_bytes[a] > (1LL << 22);
+        // complex128 lines of the smooth lengths, bound by the FP64 pipe, gain nothing from tiles in
+        // flight and lose to the persistent loop and to fewer CTAs per SM.  Measured at every smooth length,
+        // plain kernels against pipelined ones: 25 points N1 1704 -> 1592 us, 200 points 0.965, 360 points
+        // 0.93 (and three Poisson kernels against the fused one 0.88 to 1.00: 30 points 7200 -> 6570 us); above
+        // 400 points both ways (0.90 at 640 points, 1.03 at 1000), left pipelined
+        const bool plain = elem == 16 && ks->smooth && ks->n <= 400;
         ap.pipe_avail = !far;
-        ap.pipe = !far;
+        ap.pipe = !far && !plain;
         ap.rp_slots = 0;
         ap.rp_early = false;
         if (ks->pipe_rp[0] && ks->pipe_smem_rp <= max_smem) {

@@ -254,6 +254,7 @@ struct KernelSet {
     int max_threads;               // largest CTA the kernels were compiled for
     bool generic;
     bool split;                    // radix-16 passes on the tensor cores
+    bool smooth;                   // a family of AFFT_SMOOTH_PLANS
     bool contig_pad;               // the contiguous kernels pad their shared tile (contig_tile_elems)
     const void *pipe[PIPE_COUNT];  // null when the family has no pipelined strided kernel
     const void *pipe_blk[2];       // its blocked-row TMA variants ([0] forward, [1] backward)

@@ -1084,6 +1084,7 @@ template <class F, typename V, bool Contig = true> KernelSet kernel_set(int n, i
     k.max_threads = F::template threads<V>();
     k.generic = F::generic;
     k.split = F::split;
+    k.smooth = F::plan::smooth;
     k.contig_pad = F::plan::pad;
     if constexpr (F::generic) {
         if constexpr (!F::mixed || sizeof(V) == 8) {

@@ -819,23 +819,37 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
 // complex64 304-367 -> 66-75 us (230 MB through HBM: 34 us), the N1 stage of 320 x 300 x 500 r2c
 // 393 -> 91 us, its r2c stage 469 -> 100 us; complex128 (bound by the FP64 pipe) 250 -> 186-232 us
 // a stage of 180 x 200 x 216 r2c, from fewer inter-pass twiddles.
-// Above 1024 points lines are rare enough to stay with the generic kernels.  (Four groups: one
+// Above 1024 points lines are rare enough to stay with the generic kernels.  (Groups: one
 // translation unit each per precision.)
 #define AFFT_SMOOTH_PLANS_A(X)                                                                      \
-    X(18, 3, 6) X(20, 5, 4) X(36, 9, 4) X(81, 9, 9) X(90, 10, 9) X(200, 5, 5, 8) X(243, 9, 3, 9)    \
+    X(18, 3, 6) X(20, 5, 4) X(36, 9, 4) X(90, 10, 9) X(200, 5, 5, 8) X(243, 9, 3, 9)                \
     X(250, 5, 5, 10) X(320, 5, 8, 8) X(450, 9, 5, 10) X(500, 10, 5, 10) X(625, 5, 5, 5, 5)          \
     X(640, 8, 8, 10) X(675, 15, 5, 9) X(750, 15, 5, 10) X(810, 10, 9, 9)
 #define AFFT_SMOOTH_PLANS_B(X)                                                                      \
-    X(6, 6) X(9, 9) X(27, 9, 3) X(30, 5, 6) X(72, 9, 8) X(125, 5, 5, 5) X(135, 15, 9)               \
-    X(180, 15, 12) X(216, 6, 9, 4) X(240, 16, 15) X(270, 6, 9, 5) X(432, 6, 9, 8)                   \
-    X(480, 8, 6, 10) X(540, 6, 9, 10) X(729, 9, 9, 9) X(864, 9, 8, 12) X(960, 8, 10, 12)
+    X(6, 6) X(9, 9) X(27, 9, 3) X(30, 5, 6) X(54, 9, 6) X(72, 9, 8) X(125, 5, 5, 5) X(135, 15, 9)   \
+    X(180, 15, 12) X(216, 6, 9, 4) X(240, 16, 15) X(270, 6, 9, 5) X(480, 8, 6, 10)                  \
+    X(540, 6, 9, 10) X(864, 9, 8, 12) X(960, 8, 10, 12)
 #define AFFT_SMOOTH_PLANS_C(X)                                                                      \
-    X(3, 3) X(12, 12) X(25, 5, 5) X(45, 9, 5) X(50, 10, 5) X(75, 15, 5) X(108, 9, 12)               \
-    X(225, 15, 15) X(288, 8, 6, 6) X(324, 6, 9, 6) X(360, 9, 5, 8) X(400, 5, 8, 10)                 \
-    X(486, 6, 9, 9) X(648, 9, 8, 9) X(720, 9, 8, 10) X(900, 10, 9, 10) X(972, 9, 9, 12)
+    X(3, 3) X(12, 12) X(25, 5, 5) X(50, 10, 5) X(108, 9, 12) X(225, 15, 15) X(288, 8, 6, 6)         \
+    X(324, 6, 9, 6) X(400, 5, 8, 10) X(486, 6, 9, 9) X(720, 9, 8, 10) X(900, 10, 9, 10)             \
+    X(972, 9, 9, 12)
 #define AFFT_SMOOTH_PLANS_D(X)                                                                      \
-    X(5, 5) X(10, 10) X(15, 15) X(40, 8, 5) X(54, 9, 6) X(100, 10, 10) X(144, 16, 9)                \
-    X(150, 15, 10) X(162, 6, 9, 3) X(300, 5, 6, 10) X(375, 15, 5, 5) X(405, 9, 5, 9)                \
-    X(576, 9, 8, 8) X(600, 6, 10, 10) X(768, 8, 8, 12) X(800, 8, 10, 10) X(1000, 10, 10, 10)
+    X(5, 5) X(10, 10) X(15, 15) X(40, 8, 5) X(100, 10, 10) X(144, 16, 9) X(150, 15, 10)             \
+    X(162, 6, 9, 3) X(300, 5, 6, 10) X(375, 15, 5, 5) X(405, 9, 5, 9) X(600, 6, 10, 10)             \
+    X(768, 8, 8, 12) X(800, 8, 10, 10) X(1000, 10, 10, 10)
+// Lengths with a sequence per precision.  Complex128 lines are bound by the FP64 pipe, which costs a warp
+// the same for one lane as for 32, so a few wide butterflies cost more than their operations: 45 = 9 5 has
+// 40 radix-9 butterflies in a tile of eight columns, 62% of two warps' lanes.  Operations times lanes
+// issued order the sequences as measured.  N1 stages of 30 M points, generic kernels (one pass per factor)
+// / complex64 sequence / this: 45 1407 1652 1222 us, 75 1507 1691 1438, 81 1519 1769 1510, 360 2154 1973 1640,
+// 432 1869 1797 1569, 576 1773 1818 1537, 648 2437 2137 1912, 729 2670 2567 2298; c2r lines of 2 x 648 2745 2908
+// 2745, of 2 x 729 2976 3277 2953.  Errors against 64 bits stay between 1.6 and 3.1e-16 (81 = 3 3 3 3 measured
+// 1388 us but 2.5e-16 against 2.1 and 2.3e-16 for 9 9 and 9 3 3).
+#define AFFT_SMOOTH_PLANS_F32(X)                                                                    \
+    X(45, 9, 5) X(75, 15, 5) X(81, 9, 9) X(360, 9, 5, 8) X(432, 6, 9, 8)                            \
+    X(576, 9, 8, 8) X(648, 9, 8, 9) X(729, 9, 9, 9)
+#define AFFT_SMOOTH_PLANS_F64(X)                                                                    \
+    X(45, 15, 3) X(75, 5, 5, 3) X(81, 9, 3, 3) X(360, 15, 6, 4)                                     \
+    X(432, 12, 6, 6) X(576, 12, 12, 4) X(648, 12, 9, 6) X(729, 3, 3, 3, 3, 3, 3)
 
 }  // namespace afft
