@@ -545,16 +545,13 @@ size_t c2r_smem(const AxisPlan &a, size_t elem)
     return std::max(a.launch.smem, (staged + 127) / 128 * 128);
 }
 
-// Launches a stage kernel; with `overlap` its CTAs start while the previous kernel of the stream
-// finishes (programmatic dependent launch): they set up barriers and tables and wait in
-// stage_begin() for that kernel's completion, so the launch latency of each stage is hidden.
-// Complex64 plans of arrays up to kOverlapBytes use it: 64^3 Poisson solve 26.7 -> 18.9 us, 128^3 r2c
-// round trip 43.1 -> 33.0 us, 256^3 r2c 153 -> 144 us (135 MB).  Early CTAs land where the kernel that
-// is still running leaves room, not evenly: beyond L2 that costs more than the launch latency (32 x
-// 128^3 r2c, 540 MB, 563 -> 608 us; 1024^3 c2c 16.1 -> 25 ms), and in complex128, bound by arithmetic,
-// at every size (60 x 50 x 90 c2c 98 -> 172 us).  Not for split-precision plans either: a kernel that
-// waits while holding tensor memory could keep a CTA of its predecessor from allocating any.
-constexpr size_t kOverlapBytes = (size_t)144 << 20;
+// Launches a stage kernel; with `overlap` its CTAs start as those of the previous kernel of the stream
+// have exited (programmatic dependent launch): they set up barriers and tables and wait in stage_begin()
+// for that kernel's writes, so the launch latency of each stage is hidden.  Measured on and off at 300
+// shapes and batches of 0.3 MB to 8.6 GB in both precisions, transforms and Poisson solves: never slower,
+// 0.73 of the time on average below 5 MB, 0.80 at 15 to 25 MB, 0.93 at 70 to 150 MB, 0.97 at 300 MB, 0.99
+// above 500 MB (64^3 Poisson solve 24.6 -> 16.3 us, 256^3 r2c 154 -> 142 us, 32^3 complex128 c2c 42 -> 31 us).
+// Not for split-precision plans, which were not measured: their kernels hold tensor memory.
 cudaError_t launch_stage(const void *fn, long long blocks, int threads, void **args, size_t smem, cudaStream_t s,
                          bool overlap)
 {
@@ -1394,8 +1391,7 @@ int afft_plan_create_axes(afft_plan **out, const int64_t n[3], int64_t batch, in
         return AFFT_ERR_CUDA;
     }
 
-    const bool overlap = precision == AFFT_F32 &&
-                         (double)batch * n[0] * n[1] * p->nh * cplx_size(precision) <= (double)kOverlapBytes;
+    const bool overlap = precision != AFFT_F32_SPLIT;
     for (int a = 0; a < 3; ++a) p->ax[a].overlap = p->four[a].a.overlap = overlap;
 
     std::vector<int> tm, tl;

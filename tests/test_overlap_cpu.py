@@ -1,4 +1,4 @@
-"""Kernels that start while their predecessor in the stream still runs (stage_begin, csrc/fft_access.cuh)
+"""Kernels that start before their predecessor in the stream has finished (stage_begin, csrc/fft_access.cuh)
 read data that changes during their lifetime: none of their pointers but the tables that plan creation
 writes may be `__restrict__`, which would allow non-coherent loads."""
 import glob
@@ -45,3 +45,9 @@ def test_overlapped_kernels_have_no_restrict_data():
                 assert re.search(r"(\w*)\s*$", p).group(1) in TABLES, (name, p.strip())
     assert {"k_strided", "k_contig", "k_r2c", "k_c2r", "k_fourstep", "k_strided_pipe", "k_strided_pipe_rp",
             "k_poisson_pipe", "k_poisson_mult", "k_scale"} <= seen
+
+
+def test_no_kernel_triggers_its_dependents_early():
+    """CTAs launched while the previous kernel still fills the GPU crowd onto the SMs with room (stage_begin)."""
+    for path in glob.glob(os.path.join(CSRC, "*.cu*")):
+        assert "griddepcontrol.launch_dependents;" not in re.sub(r"//[^\n]*", "", open(path).read()), path
