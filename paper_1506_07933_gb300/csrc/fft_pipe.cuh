@@ -156,10 +156,16 @@ template <class P, typename V, int PairValues = P::smooth ? 20 : 16, bool RowPai
         for (int r : {Rs...}) e = e && !pairs(r);
         return e;
     }
-    // thread map of the single-column passes (DefineBoth; row-pair tiles with only such passes, all
-    // of them exact -- 256 points -- measured faster without: 194 against 200 us on N1 of 8 x 256^3,
-    // while 128 = 16 x 8 gains: 101 -> 93 us on N1 of 32 x 128^3)
-    using map = MapLineFastC<lg, !(RowPairs && exact_for(typename P::seq{}) && singles_for(typename P::seq{}))>;
+    // thread map of the single-column passes (DefineBoth).  Defined: complex128 and the smooth lengths;
+    // row-pair tiles, unless all their passes are single-column and exact (256 points measured faster without:
+    // 194 against 200 us on N1 of 8 x 256^3, while 128 = 16 x 8 gains: 101 -> 93 us on N1 of 32 x 128^3); and of
+    // the other complex64 tiles the exact ones of narrower rows, 1024 points (N1 of 1024^3 c2c 2.91 -> 2.69 ms).
+    // The rest lose: N1 of 48 points in rows of 24 56 -> 67 us, 80 points 56 -> 65 us, 384^3 c2c 163 -> 168 us.
+    static constexpr bool define_singles =
+        sizeof(V) == 16 || P::smooth ||
+        (RowPairs ? !(exact_for(typename P::seq{}) && singles_for(typename P::seq{}))
+                  : lines < row_lines && exact_for(typename P::seq{}));
+    using map = MapLineFastC<lg, define_singles>;
     using seq = typename P::seq;
     static constexpr int npass = P::npass;
     static constexpr int tile = P::n * lines;                       // complex elements per tile

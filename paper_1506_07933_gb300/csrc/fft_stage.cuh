@@ -56,10 +56,10 @@ struct MapButterflyFast {  // contiguous stage: consecutive threads walk along a
 // Whether a pass defines its values on both sides of `this thread has a butterfly`.  Left undefined
 // on the idle side, they are live around the tile loop of a persistent kernel (that side carries
 // the last tile's): 20 to 60 registers, and spills where those are short.  The persistent strided
-// kernels and the multi-plan executor define them (complex128 512^3 r2c N1/N0 1137/1105 ->
-// 1041/1014 us, 192 points 156/148 -> 131/122 us); in one-tile kernels, and in the column-pair passes
-// of complex64 tiles (pair_pass), whose registers suffice, the second branch only costs (r2c lines
-// of 320 x 300 x 500 100 -> 118 us, N0 stage of 16 x 160^3 87 -> 90 us).
+// kernels of complex128 and of the smooth lengths and the multi-plan executor define them (complex128
+// 512^3 r2c N1/N0 1137/1105 -> 1041/1014 us, 192 points 156/148 -> 131/122 us); in one-tile kernels, and in
+// most complex64 tiles (define_singles and define_pairs in PipeShape), whose registers suffice, the second
+// branch only costs (r2c lines of 320 x 300 x 500 100 -> 118 us, N0 stage of 16 x 160^3 87 -> 90 us).
 template <class Map, typename V> struct DefineBoth { static constexpr bool value = false; };
 
 // ------------------------------------------------------ one radix pass ------
