@@ -148,8 +148,9 @@ const KernelSet *lookup_kernels(int precision, int64_t n, bool contiguous)
             if (const KernelSet *k = smooth_kernels_f32((int)n)) return k;
         return generic_kernels_split();
     }
-    if (precision == AFFT_F64 && !contiguous)
-        if (const KernelSet *k = strided_kernels_f64((int)n)) return k;
+    if (!contiguous)
+        if (const KernelSet *k = precision == AFFT_F64 ? strided_kernels_f64((int)n) : strided_kernels_f32((int)n))
+            return k;
     const KernelSet *k = precision == AFFT_F64 ? spec_kernels_f64((int)n) : spec_kernels_f32((int)n);
     if (!k) k = precision == AFFT_F64 ? smooth_kernels_f64((int)n) : smooth_kernels_f32((int)n);
     if (k) return k;

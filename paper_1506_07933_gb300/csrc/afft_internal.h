@@ -287,8 +287,9 @@ struct KernelSet {
 // Specialised kernels for line length n, or nullptr.
 const KernelSet *spec_kernels_f32(int n);
 const KernelSet *spec_kernels_f64(int n);
-// The strided kernels of AFFT_STRIDED_PLANS_F64 (lengths whose strided stages prefer another radix
-// sequence than their contiguous ones; no contiguous kernels), or nullptr.
+// The strided kernels of AFFT_STRIDED_PLANS_F32 / _F64 (lengths whose strided stages prefer another
+// radix sequence than their contiguous ones; no contiguous kernels), or nullptr.
+const KernelSet *strided_kernels_f32(int n);
 const KernelSet *strided_kernels_f64(int n);
 // The families of AFFT_SMOOTH_PLANS (the other 2/3/5-smooth lengths up to 1024), or nullptr.
 const KernelSet *smooth_kernels_f32(int n);

@@ -785,16 +785,20 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
 // each length; complex128 (float-float, four registers per value) wants fewer values per thread, so
 // the two precisions differ.  Complex64, previous -> this: 60 = 4 3 5 -> 10 6 (c2c N2/N1/N0 of 64
 // fields 67/38/33 -> 45/35/31 us), 120 = 8 3 5 -> 8 15 (N1/N0 49/36 -> 40/34 us), 160 = 8 4 5 ->
-// 10 16 (121/90 -> 110/87 us), 192 = 8 8 3 -> 12 16 (94/79 -> 90/76 us, r2c of 384^3 102 -> 94 us).
+// 10 16 (strided stages, 121/90 -> 110/87 us), 192 = 8 8 3 -> 12 16 (94/79 -> 90/76 us, r2c of 384^3 102 -> 94 us).
 // Complex128: 384 = 16 8 3 -> 6 8 8 (611/578 -> 465/446 us, its fused Poisson stage 1879 -> 744 us:
 // radix 16 spills there), 1024 = 16 8 8 -> 8 8 4 4 (N1 of 64 x 1024^2 c2c 1213 -> 1126 us).  Measured
 // the same or slower: 128 = 8 4 4, 256 = 8 8 4, 384 = 6 8 8 and 1024 = 8 8 16 in complex64; 60 = 10 6,
 // 96 = 8 12, 120 = 8 15, 160 = 16 10 and 192 = 12 16 in complex128; 48 = 8 6 and 80 = 8 10 in either.
 #define AFFT_LINE_PLANS(X)                                                                          \
     X(1) X(2, 2) X(4, 4) X(8, 8) X(16, 16) X(24, 8, 3) X(32, 8, 4) X(48, 16, 3) X(60, 10, 6)        \
-    X(64, 8, 8) X(80, 16, 5) X(96, 8, 4, 3) X(120, 8, 15) X(128, 16, 8) X(160, 10, 16)              \
+    X(64, 8, 8) X(80, 16, 5) X(96, 8, 4, 3) X(120, 8, 15) X(128, 16, 8) X(160, 16, 10)              \
     X(192, 12, 16) X(256, 16, 16) X(384, 16, 8, 3) X(512, 8, 8, 8) X(1024, 16, 8, 8)                \
     X(2048, 16, 16, 8) X(4096, 16, 16, 16)
+// complex64 lengths whose strided stages are faster with another sequence than their contiguous ones (160 =
+// 16 10: r2c lines of 3000 x 64 x 320 142 -> 99 us, with 8 4 5 130 us, c2c lines 121 -> 102 us; but the N1 stage of
+// 3000 x 160 x 160 194 -> 203 us)
+#define AFFT_STRIDED_PLANS_F32(X) X(160, 10, 16)
 // complex128, in five groups (the slowest instantiations to compile: one translation unit each)
 #define AFFT_LINE_PLANS_F64_A(X)                                                                    \
     X(1) X(2, 2) X(4, 4) X(8, 8) X(16, 16) X(24, 8, 3) X(32, 8, 4) X(48, 16, 3) X(60, 4, 3, 5) X(64, 8, 8)

@@ -1,5 +1,6 @@
 // kernels_f32.cu -- instantiates the stage kernels for float2: one specialised
-// family per line length of AFFT_LINE_PLANS, plus the generic family.
+// family per line length of AFFT_LINE_PLANS, the strided-only sets of
+// AFFT_STRIDED_PLANS_F32, and the generic family.
 #include "kernel_tables.cuh"
 
 namespace afft {
@@ -9,6 +10,17 @@ namespace afft {
 const KernelSet *spec_kernels_f32(int n)
 {
     static const KernelSet table[] = {AFFT_LINE_PLANS(AFFT_X)};
+    return find_set(table, n);
+}
+
+#undef AFFT_X
+#define AFFT_X(N, ...)                                                                               \
+    afft::kernel_set<afft::Spec<afft::LinePlan<N, ##__VA_ARGS__>>, float2, false>(                    \
+        N, afft::LinePlan<N, ##__VA_ARGS__>::npass, afft::RadicesOf<afft::LinePlan<N, ##__VA_ARGS__>>::value),
+
+const KernelSet *strided_kernels_f32(int n)
+{
+    static const KernelSet table[] = {AFFT_STRIDED_PLANS_F32(AFFT_X)};
     return find_set(table, n);
 }
 

@@ -107,3 +107,13 @@ def test_poisson_every_n0_length(n):
                 assert p.device_status() == 0
             err = oracle.rel_l2(u.cpu().numpy(), oracle.poisson(f.astype(np.float64)))
             assert err <= (2e-6 if prec == "f32" else 1e-12), (shape, prec, err)
+
+
+def test_length_with_a_strided_and_a_contiguous_sequence():
+    """160 points in complex64: strided stages 10 x 16, contiguous lines 16 x 10."""
+    check((160, 4, 10), "c2c", "f32", 1)
+    check((2, 160, 25), "c2c", "f32", 2)
+    check((3, 160, 160), "c2c", "f32", 3)
+    check((2, 5, 320), "r2c", "f32", 4)
+    with afft.Plan((160, 160, 160), "c2c", "f32") as p:
+        assert p.describe()["radix"] == ["10x16", "10x16", "16x10"]
