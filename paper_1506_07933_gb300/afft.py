@@ -355,10 +355,10 @@ class Plan:
     def tune(self, stream=None, cache: str = None) -> bool:
         """Autotune the launch configuration on temporary buffers (synchronises).  With `cache`
         (a JSON file), a choice stored there for this plan's key (shape, kind, precision, batch,
-        GPU name) is applied instead of tuning, and a new one is stored.  Returns True when the
-        choice came from the cache."""
+        GPU name, KERNEL_TABLES) is applied instead of tuning, and a new one is stored.  Returns
+        True when the choice came from the cache."""
         key = tuning_key(self.shape, self.kind, self.precision, self.batch,
-                         torch.cuda.get_device_name(self.device)) if cache else None
+                         torch.cuda.get_device_name(self.device), KERNEL_TABLES) if cache else None
         if cache:
             cfg = tuning_cache_lookup(cache, key)
             if cfg is not None:
@@ -517,12 +517,20 @@ class Queue:
             pass
 
 
-def tuning_key(shape, kind, precision, batch, gpu_name: str) -> str:
-    """Cache key of a plan's tuned configuration."""
+# Version of what a tuned configuration was measured on: radix sequences, tile shapes and default rules
+# (csrc).  A change there makes stored choices stale -- early release stored for 120-point rows as
+# 8 x 3 x 5 takes 53 us where 8 x 15 without it takes 39 -- so it takes a new number, and entries stored
+# under another (or none) are not found: the plan tunes again.
+KERNEL_TABLES = 2
+
+
+def tuning_key(shape, kind, precision, batch, gpu_name: str, tables=None) -> str:
+    """Cache key of a plan's tuned configuration (tables: the version of the kernel tables)."""
     kinds = {v: k for k, v in KINDS.items()}
     precs = {v: k for k, v in PRECISIONS.items()}
-    return "%s/%s/%s/batch%d/%s" % ("x".join(str(int(n)) for n in shape), kinds.get(kind, kind),
-                                    precs.get(precision, precision), int(batch or 1), gpu_name)
+    key = "%s/%s/%s/batch%d/%s" % ("x".join(str(int(n)) for n in shape), kinds.get(kind, kind),
+                                   precs.get(precision, precision), int(batch or 1), gpu_name)
+    return key if tables is None else "%s/tables%d" % (key, tables)
 
 
 def tuning_cache_lookup(path: str, key: str):
