@@ -230,22 +230,20 @@ bool shape_strided(const StageDesc &d, long long outer, long long W, size_t elem
     }
 }
 
-constexpr int kSMs = 152;   // GB300
-
 // Contiguous stage: whole lines, about `target` complex points per CTA
-// (0: 4096 for complex64, 2048 for complex128; the autotuner may pick others).
+// (0: 4096 for complex64, 2048 for complex128; the autotuner may pick others).  sms: the device's SMs.
 // even_lines: an even count where possible, so that every CTA's run of lines of
 // an odd number of complex64 elements starts 16-byte aligned (the c2r kernel
 // then stages it with 16-byte copies).
 bool shape_contig(const StageDesc &d, const KernelSet *ks, long long nlines, size_t elem, size_t max_smem,
-                  Launch &L, int target = 0, bool even_lines = false)
+                  int sms, Launch &L, int target = 0, bool even_lines = false)
 {
     if (target <= 0) {
         target = elem == 8 ? 4096 : 2048;
         // small complex64 arrays: down to one warp's worth of points per CTA, so that all SMs have
         // work (the float-float kernels are bound by instruction fetch there and lose: 16 x 32 x 20 x
         // 32 FP64 c2c 83 -> 98 us)
-        while (elem == 8 && target > 512 && nlines * d.n < 2LL * kSMs * target) target /= 2;
+        while (elem == 8 && target > 512 && nlines * d.n < 2LL * sms * target) target /= 2;
     }
     int lines = std::max(1, target / std::max(1, d.n));
     lines = (int)std::min<long long>(lines, std::max(1LL, nlines));
@@ -269,7 +267,7 @@ bool shape_contig(const StageDesc &d, const KernelSet *ks, long long nlines, siz
             int rmax = 1;
             for (int p = 0; p < d.npass; ++p) rmax = std::max(rmax, d.radix[p]);
             L.c2r_threads = elem == 16 && !ks->generic && rmax <= 8 ? std::min(2 * thr, ks->max_threads) : thr;
-            if (!ks->generic && !ks->split && L.blocks <= 2 * kSMs) {
+            if (!ks->generic && !ks->split && L.blocks <= 2 * sms) {
                 L.threads = std::min(2 * thr, ks->max_threads);
                 L.c2r_threads = std::max(L.c2r_threads, L.threads);
             }
@@ -505,7 +503,7 @@ int plan_shapes(afft_plan *p)
         AxisPlan &ap = p->ax[a];
         bool ok;
         if (a == 2 && !f.on)
-            ok = shape_contig(z.desc, z.ks, B * n0 * n1, elem, budget(z), z.launch, 0,
+            ok = shape_contig(z.desc, z.ks, B * n0 * n1, elem, budget(z), sms, z.launch, 0,
                               p->kind == AFFT_R2C && (nh & 1));
         else ok = shape_strided(ap.desc, outer[a], width[a] * (f.on ? f.na : 1), elem, ap.ks->max_threads,
                                 budget(ap), ap.launch);
@@ -549,9 +547,10 @@ size_t c2r_smem(const AxisPlan &a, size_t elem)
 // Launches a stage kernel; with `overlap` its CTAs start as those of the previous kernel of the stream
 // have exited (programmatic dependent launch): they set up barriers and tables and wait in stage_begin()
 // for that kernel's writes, so the launch latency of each stage is hidden.  Measured on and off at 300
-// shapes and batches of 0.3 MB to 8.6 GB in both precisions, transforms and Poisson solves: never slower,
-// 0.73 of the time on average below 5 MB, 0.80 at 15 to 25 MB, 0.93 at 70 to 150 MB, 0.97 at 300 MB, 0.99
-// above 500 MB (64^3 Poisson solve 24.6 -> 16.3 us, 256^3 r2c 154 -> 142 us, 32^3 complex128 c2c 42 -> 31 us).
+// shapes and batches of 0.3 MB to 8.6 GB (spectrum) in both precisions, transforms and Poisson solves: never
+// slower; complex64 0.70 of the time on average below 15 MB, 0.78 at 15 to 25 MB, 0.88 at 35 to 46 MB, 0.93
+// at 70 to 150 MB, 0.98 at 300 MB, 0.99 above 500 MB; complex128, bound by arithmetic, 0.8 below 8 MB and 0.99
+// from 100 MB (64^3 Poisson solve 24.6 -> 17 us, 256^3 r2c 154 -> 139 us, 32^3 complex128 c2c 42 -> 31 us).
 // Not for split-precision plans, which were not measured: their kernels hold tensor memory.
 cudaError_t launch_stage(const void *fn, long long blocks, int threads, void **args, size_t smem, cudaStream_t s,
                          bool overlap)
@@ -1281,7 +1280,9 @@ bool reshape_contig(afft_plan *p, int target)
     const size_t budget = z.ks->generic ? (size_t)max_smem : (size_t)std::min(max_smem, 112 * 1024);
     Launch L;
     const bool even = p->kind == AFFT_R2C && ((p->n[2] / 2 + 1) & 1);
-    if (!shape_contig(z.desc, z.ks, p->batch * p->n[0] * p->n[1], sizeof(V), budget, L, target, even))
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    if (!shape_contig(z.desc, z.ks, p->batch * p->n[0] * p->n[1], sizeof(V), budget, sms, L, target, even))
         return false;
     z.launch = L;
     p->contig_target = target;

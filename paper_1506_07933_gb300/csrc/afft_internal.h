@@ -60,7 +60,8 @@ __host__ __device__ inline long long blocked_line(const StageDesc &d, long long 
 }
 
 // Butterflies a thread carries per pass for radix R: at most 16 complex
-// values in registers (15 for radix 3 and 5).  The host picks the thread
+// values in registers (15 for radix 3 and 5; the pipelined tiles have counts of their own, up to 20
+// values, see PipeShape).  The host picks the thread
 // count so that threads * bmax(R) covers every butterfly of every pass.
 __host__ __device__ constexpr int bmax_for_radix(int r)
 {

@@ -42,8 +42,8 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 // No kernel triggers its dependents (griddepcontrol.launch_dependents): its CTAs do so by exiting, so the
 // next kernel's CTAs start on a GPU that is all but empty and spread over every SM.  Triggered early they
 // land where the running kernel leaves room, and stay there: 2048 x 32 x 32 r2c, whose N0 stage has
-// 136 CTAs, ran 1.27 times as long as without overlap, 24 x 128^3 r2c 1.08 and its batches of 46 to 150 MB up
-// to 1.25 times; by exit they run 0.76 and 0.97 times as long.
+// 136 CTAs, ran 1.27 times as long as without overlap (0.76 by exit), 5 x 384 x 32 x 32 r2c 1.08 (0.75),
+// batches of 46 to 150 MB up to 1.25 times.
 __device__ __forceinline__ void stage_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // mbarriers (shared::cta) for the asynchronous copies of the tensor-memory

@@ -821,7 +821,7 @@ __global__ void k_poisson_mult(V *x, long long planes, int n0, int n1, int nhp, 
 // shared-memory round trip per pass plus two to stage the tile, with run-time lengths in every
 // index and one tile per CTA in flight.  Measured, generic kernels -> these: a c2c stage of 243^3
 // complex64 304-367 -> 66-75 us (230 MB through HBM: 34 us), the N1 stage of 320 x 300 x 500 r2c
-// 393 -> 91 us, its r2c stage 469 -> 100 us; complex128 (bound by the FP64 pipe) 250 -> 186-232 us
+// 393 -> 91 us, its r2c stage 469 -> 100 us; complex128 (bound by the FP64 pipe) 250 -> 180-230 us
 // a stage of 180 x 200 x 216 r2c, from fewer inter-pass twiddles.
 // Above 1024 points lines are rare enough to stay with the generic kernels.  (Groups: one
 // translation unit each per precision.)
