@@ -242,8 +242,9 @@ bool shape_contig(const StageDesc &d, const KernelSet *ks, long long nlines, siz
         target = elem == 8 ? 4096 : 2048;
         // small complex64 arrays: down to one warp's worth of points per CTA, so that all SMs have
         // work (the float-float kernels are bound by instruction fetch there and lose: 16 x 32 x 20 x
-        // 32 FP64 c2c 83 -> 98 us)
-        while (elem == 8 && target > 512 && nlines * d.n < 2LL * sms * target) target /= 2;
+        // 32 FP64 c2c 83 -> 98 us; split-precision ones would leave tcgen05, whose passes take 128
+        // butterflies at a time: 64^3 c2c 57 -> 76 us)
+        while (elem == 8 && !ks->split && target > 512 && nlines * d.n < 2LL * sms * target) target /= 2;
     }
     int lines = std::max(1, target / std::max(1, d.n));
     lines = (int)std::min<long long>(lines, std::max(1LL, nlines));

@@ -145,3 +145,11 @@ def test_batched_split_plan_and_poisson():
         torch.cuda.synchronize()
     for b in range(B):
         report("poisson batched split [%d]" % b, oracle.rel_l2(got[b].cpu().numpy(), us[b]))
+
+
+def test_small_arrays_keep_tiles_the_tensor_cores_take():
+    """tcgen05 passes take 128 butterflies at a time: small split-precision arrays keep contiguous tiles of
+    4096 points (smaller ones, which complex64 plans use there, fell back to mma.sync: 64^3 57 -> 76 us)."""
+    for n in (32, 64, 128):
+        with afft.Plan((n, n, n), "c2c", "f32_split") as p:
+            assert p.describe()["contig_lines"] * n == 4096
